@@ -134,7 +134,8 @@ typedef struct {
     uint8_t* klass;            /* CS_SECURE .. CS_EIG_FAIL */
     uint8_t* severe;           /* S_c in {0, 1} */
     int16_t* n_islands;        /* number of islands of the post-contingency network */
-    int16_t* opf_iters;        /* interior-point iterations taken (0 if not run) */
+    int16_t* opf_iters;        /* interior-point iterations taken (0 if not run); the cap for a scenario
+                                  stopped because it can no longer converge within it */
     double* cost;              /* OPF cost, $/h (NaN if not converged) */
     double* max_re;            /* largest real part, structural zero mode removed (NaN if not run) */
     double* min_zeta;          /* smallest damping ratio (NaN if not run) */
