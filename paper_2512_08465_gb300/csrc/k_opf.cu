@@ -59,7 +59,7 @@ namespace {
 constexpr int kThreads = CS_OPF_THREADS;   // threads per scenario CTA
 constexpr int kCtasPerSm = CS_OPF_CTAS;    // resident CTAs per SM the register budget is sized for
 constexpr int kWarps = kThreads / 32;
-constexpr int kRec = 46;     // doubles per branch record
+constexpr int kRec = 34;     // doubles per branch record
 constexpr double kXi = 0.99995;
 constexpr double kSigma = 0.1;
 constexpr double kLimitTol = 1e-6;
@@ -72,23 +72,46 @@ constexpr int kPanel = 8;                    // panel width of the dense fallbac
 constexpr int kGmresM = 8;                   // GMRES iterations per Newton solve (at most)
 constexpr int kRedMax = kGmresM + 1 > 10 ? kGmresM + 1 : 10;   // values per block reduction (at most)
 
-// record layout
-constexpr int R_DSF = 0, R_DST = 8, R_GF = 16, R_GT = 20, R_H = 24, R_LG = 34, R_NG = 38, R_SF = 42, R_ST = 44;
+// Branch record.  Every branch quantity depends on the two end angles through theta = Va_f -
+// Va_t alone, so derivatives are kept by (theta, Vm_f, Vm_t); those by Va_t are those by theta with
+// the sign changed.  R_H: second derivatives (theta theta, theta f, theta t, f f, f t, t t);
+// R_DF, R_DT: complex derivatives of the powers at the f and t ends; R_G: gradients of the two
+// |S|^2; R_L, R_N: contributions to the Lagrangian gradient and to N; R_S: S_f, S_t.
+constexpr int R_H = 0, R_DF = 6, R_DT = 12, R_G = 18, R_L = 24, R_N = 27, R_S = 30;
 
-__device__ __forceinline__ int hidx(int p, int q) {
-    if (p > q) { int t = p; p = q; q = t; }
-    // (0,0)0 (0,1)1 (0,2)2 (0,3)3 (1,1)4 (1,2)5 (1,3)6 (2,2)7 (2,3)8 (3,3)9
-    const int base[4] = {0, 4, 7, 9};
-    return base[p] + (q - p);
+// x with its sign changed (on the integer pipe)
+__device__ __forceinline__ double neg(double x) {
+    return __longlong_as_double(__double_as_longlong(x) ^ (long long)0x8000000000000000ull);
+}
+__device__ __forceinline__ bool non_finite(double x) { return (__double2hiint(x) & 0x7ff00000) == 0x7ff00000; }
+
+// Maxima of non-negative doubles run on the integer pipe: as 64-bit integers they have the same
+// order, +0 below everything, NaN above everything (a NaN in one of the maxima makes the
+// iteration fail, as it should).  An FP64 comparison would hold the sub-partition's FP64 pipe for
+// as long as a multiply-add does.
+typedef unsigned long long key_t64;
+__device__ __forceinline__ key_t64 abs_key(double x) {
+    return (key_t64)__double_as_longlong(x) & 0x7fffffffffffffffull;
+}
+__device__ __forceinline__ key_t64 pos_key(double x) {      // negative values count as 0
+    const long long v = __double_as_longlong(x);
+    return v < 0 ? 0ull : (key_t64)v;
+}
+__device__ __forceinline__ double key_value(key_t64 k) { return __longlong_as_double((long long)k); }
+__device__ __forceinline__ key_t64 warp_max_key(key_t64 k) {
+    const unsigned hi = (unsigned)(k >> 32), lo = (unsigned)k;
+    const unsigned mh = __reduce_max_sync(0xffffffffu, hi);
+    const unsigned ml = __reduce_max_sync(0xffffffffu, hi == mh ? lo : 0u);
+    return ((key_t64)mh << 32) | ml;
 }
 
 struct Lay {
     // bus
-    int Va, Vm, lP, lQ, zu, zl, muu, mul, gP, gQ, LxVa, LxVm, NVa, NVm, DP, DQ, rP, rQ, dzu, dzl, dmuu, dmul;
+    int Va, Vm, lP, lQ, zu, zl, rzu, rzl, muu, mul, gP, gQ, NVa, NVm, DP, DQ, rP, rQ, dzu, dzl, dmuu, dmul;
     // gen
-    int Pg, Qg, gz, gmu, gdz, gdmu, MP, MQ, NP, NQ, LxP, LxQ, dPg, dQg;
+    int Pg, Qg, gz, gmu, gdz, gdmu, grz, MP, MQ, NP, NQ, dPg, dQg;   // MP, MQ: reciprocals of the pivots
     // branch
-    int zf, zt, muf, mut, hf, ht, dzf, dzt, dmuf, dmut, rec;
+    int zf, zt, muf, mut, hf, ht, rzf, rzt, dzf, dzt, dmuf, dmut, rec;   // rz..: 1 / z
     // KKT: assembled blocks (Kb, Kd) kept for refinement, factor (Ub, Lb, Db, Di), vectors
     int Kb, Kd, Ub, Lb, Db, Di, x, bv, rv, cs, drs, dpiv;   // drs, dpiv: dense backstop's row scales, pivots
     int kv, kz, gx0, gxb, gr;   // GMRES: Krylov basis, preconditioned basis, start, best iterate, work
@@ -103,14 +126,16 @@ Lay make_layout(const DevNet& n) {
     auto take = [&](int cnt) { int r = o; o += cnt; return r; };
     int nb = n.nb, ng = n.ng, nbr = n.nbr;
     L.Va = take(nb); L.Vm = take(nb); L.lP = take(nb); L.lQ = take(nb); L.zu = take(nb); L.zl = take(nb);
-    L.muu = take(nb); L.mul = take(nb); L.gP = take(nb); L.gQ = take(nb); L.LxVa = take(nb); L.LxVm = take(nb);
+    L.muu = take(nb); L.mul = take(nb); L.gP = take(nb); L.gQ = take(nb); L.rzu = take(nb); L.rzl = take(nb);
     L.NVa = take(nb); L.NVm = take(nb); L.DP = take(nb); L.DQ = take(nb); L.rP = take(nb); L.rQ = take(nb);
     L.dzu = take(nb); L.dzl = take(nb); L.dmuu = take(nb); L.dmul = take(nb);
     L.Pg = take(ng); L.Qg = take(ng); L.gz = take(4 * ng); L.gmu = take(4 * ng); L.gdz = take(4 * ng);
     L.gdmu = take(4 * ng); L.MP = take(ng); L.MQ = take(ng); L.NP = take(ng); L.NQ = take(ng);
-    L.LxP = take(ng); L.LxQ = take(ng); L.dPg = take(ng); L.dQg = take(ng);
+    L.grz = take(4 * ng); L.dPg = take(ng); L.dQg = take(ng);
     L.zf = take(nbr); L.zt = take(nbr); L.muf = take(nbr); L.mut = take(nbr); L.hf = take(nbr); L.ht = take(nbr);
     L.dzf = take(nbr); L.dzt = take(nbr); L.dmuf = take(nbr); L.dmut = take(nbr);
+    L.rzf = take(nbr); L.rzt = take(nbr);
+    o = (o + 15) & ~15;
     L.rec = take(kRec * nbr);
     o = (o + 15) & ~15;
     L.Kb = take(16 * n.nL); L.Kd = take(16 * nb);
@@ -239,91 +264,96 @@ __device__ bool inv4(const double* A, double* Ainv, int q) {
 // One branch at the current iterate: flows, derivatives, weighted Hessian,
 // Lagrangian-gradient and N contributions.  If init, also sets z, mu of the
 // two flow rows from h (z = max(-h, 1), mu = gamma / z).
-__device__ void eval_branch(const DevNet& net, int b, double* W, const Lay& L, double gamma,
-                            bool init) {
+//
+// With theta = Va_f - Va_t, a = conj(yft) e^{j theta} and c = conj(ytf) e^{-j theta}:
+//   S_f = Vf^2 conj(yff) + Vf Vt a,   S_t = Vt^2 conj(ytt) + Vf Vt c,
+// and every derivative is one of a few products of these.  The FP64 pipe is the OPF's bound
+// (one warp instruction per 16 cycles and SM, whatever its lanes), so what counts here is the
+// number of FP64 instructions: ~200 with one sincos and two reciprocals, where the product rule
+// over four complex variables took ~1,400.  With it, the reductions' comparisons on the integer
+// pipe and stored reciprocals, 10,000 pairs (118 buses) went from 1,329 to 1,198 ms, one
+// scenario's OPF from 21.6 to 18.7 ms.
+__device__ __forceinline__ void eval_branch(const DevNet& net, int b, double* W, const Lay& L, double gamma,
+                                            bool init) {
     const int f = net.f[b], t = net.t[b];
-    double* rec = W + L.rec + (size_t)kRec * b;
     const double vf = W[L.Vm + f], vt = W[L.Vm + t];
-    double sf, cf, st, ct;
-    sincos(W[L.Va + f], &sf, &cf);
-    sincos(W[L.Va + t], &st, &ct);
-    const cplx ef = cm(cf, sf), et = cm(ct, st);
-    const cplx Vf = vf * ef, Vt = vt * et;
+    double sn, cs;
+    sincos(W[L.Va + f] - W[L.Va + t], &sn, &cs);
     const cplx yff = net.yff[b], yft = net.yft[b], ytf = net.ytf[b], ytt = net.ytt[b];
-    const cplx zero = cm(0.0, 0.0);
-    const cplx dVf[4] = {mulj(Vf), ef, zero, zero};
-    const cplx dVt[4] = {zero, zero, mulj(Vt), et};
-    const cplx If = yff * Vf + yft * Vt;
-    const cplx It = ytf * Vf + ytt * Vt;
-    cplx dIf[4], dIt[4], dSf[4], dSt[4];
-    for (int p = 0; p < 4; ++p) {
-        dIf[p] = yff * dVf[p] + yft * dVt[p];
-        dIt[p] = ytf * dVf[p] + ytt * dVt[p];
-    }
-    const cplx Sf = Vf * conj(If), St = Vt * conj(It);
-    for (int p = 0; p < 4; ++p) {
-        dSf[p] = dVf[p] * conj(If) + Vf * conj(dIf[p]);
-        dSt[p] = dVt[p] * conj(It) + Vt * conj(dIt[p]);
-    }
+    const cplx a = cm(yft.re * cs + yft.im * sn, yft.re * sn - yft.im * cs);
+    const cplx c = cm(ytf.re * cs - ytf.im * sn, neg(ytf.re * sn + ytf.im * cs));
+    const double p = vf * vt;
+    const cplx A = p * a, C = p * c;
+    const cplx Sf = cm(vf * vf * yff.re + A.re, A.im - vf * vf * yff.im);
+    const cplx St = cm(vt * vt * ytt.re + C.re, C.im - vt * vt * ytt.im);
+    // derivatives by (theta, Vm_f, Vm_t); those of S_f by theta are j A, of S_t -j C
+    const double df[6] = {neg(A.im), A.re, 2.0 * vf * yff.re + vt * a.re, vt * a.im - 2.0 * vf * yff.im,
+                          vf * a.re, vf * a.im};
+    const double dt[6] = {C.im, neg(C.re), vt * c.re, vt * c.im,
+                          2.0 * vt * ytt.re + vf * c.re, vf * c.im - 2.0 * vt * ytt.im};
     const double smax2 = net.smax2[b];
     const double hf = abs2(Sf) - smax2, ht = abs2(St) - smax2;
-    double zf, zt, muf, mut;
+    double muf, mut, rzf, rzt;
     if (init) {
-        zf = fmax(-hf, 1.0);
-        zt = fmax(-ht, 1.0);
-        muf = gamma / zf;
-        mut = gamma / zt;
+        const double zf = fmax(-hf, 1.0), zt = fmax(-ht, 1.0);
+        rzf = 1.0 / zf;
+        rzt = 1.0 / zt;
+        muf = gamma * rzf;
+        mut = gamma * rzt;
         W[L.zf + b] = zf; W[L.zt + b] = zt; W[L.muf + b] = muf; W[L.mut + b] = mut;
     } else {
-        zf = W[L.zf + b]; zt = W[L.zt + b]; muf = W[L.muf + b]; mut = W[L.mut + b];
+        rzf = 1.0 / W[L.zf + b];
+        rzt = 1.0 / W[L.zt + b];
+        muf = W[L.muf + b]; mut = W[L.mut + b];
     }
+    W[L.rzf + b] = rzf;
+    W[L.rzt + b] = rzt;
     W[L.hf + b] = hf;
     W[L.ht + b] = ht;
-    double gf[4], gt[4];
-    for (int p = 0; p < 4; ++p) {
-        gf[p] = 2.0 * (Sf.re * dSf[p].re + Sf.im * dSf[p].im);
-        gt[p] = 2.0 * (St.re * dSt[p].re + St.im * dSt[p].im);
-    }
     const double lPf = W[L.lP + f], lQf = W[L.lQ + f], lPt = W[L.lP + t], lQt = W[L.lQ + t];
-    // weights: Re(c * d2S) = lamP Re d2S + lamQ Im d2S + 2 mu Re(conj(S) d2S)
-    const cplx wf = cm(lPf, -lQf) + (2.0 * muf) * conj(Sf);
-    const cplx wt = cm(lPt, -lQt) + (2.0 * mut) * conj(St);
-    const double bf = muf / zf, bt = mut / zt;
-    // second derivatives of V: f end (0,0) -V_f, (0,1) j e_f ; t end (2,2) -V_t, (2,3) j e_t
-    for (int p = 0; p < 4; ++p) {
-        for (int q = p; q < 4; ++q) {
-            cplx d2Vf = zero, d2Vt = zero;
-            if (p == 0 && q == 0) d2Vf = -Vf;
-            if (p == 0 && q == 1) d2Vf = mulj(ef);
-            if (p == 2 && q == 2) d2Vt = -Vt;
-            if (p == 2 && q == 3) d2Vt = mulj(et);
-            const cplx d2If = yff * d2Vf + yft * d2Vt;
-            const cplx d2It = ytf * d2Vf + ytt * d2Vt;
-            const cplx d2Sf = d2Vf * conj(If) + dVf[p] * conj(dIf[q]) + dVf[q] * conj(dIf[p]) + Vf * conj(d2If);
-            const cplx d2St = d2Vt * conj(It) + dVt[p] * conj(dIt[q]) + dVt[q] * conj(dIt[p]) + Vt * conj(d2It);
-            double h = (wf * d2Sf).re + (wt * d2St).re;
-            h += 2.0 * muf * (dSf[q].re * dSf[p].re + dSf[q].im * dSf[p].im);
-            h += 2.0 * mut * (dSt[q].re * dSt[p].re + dSt[q].im * dSt[p].im);
-            h += bf * gf[p] * gf[q] + bt * gt[p] * gt[q];
-            rec[R_H + hidx(p, q)] = h;
-        }
+    double gf[3], gt[3], lg[3], ng[3];
+    const double nf = (muf * hf + gamma) * rzf, nt = (mut * ht + gamma) * rzt;
+#pragma unroll
+    for (int q = 0; q < 3; ++q) {
+        gf[q] = 2.0 * (Sf.re * df[2 * q] + Sf.im * df[2 * q + 1]);
+        gt[q] = 2.0 * (St.re * dt[2 * q] + St.im * dt[2 * q + 1]);
+        lg[q] = lPf * df[2 * q] + lQf * df[2 * q + 1] + lPt * dt[2 * q] + lQt * dt[2 * q + 1] + muf * gf[q] +
+                mut * gt[q];
+        ng[q] = nf * gf[q] + nt * gt[q];
     }
-    const double nf = (muf * hf + gamma) / zf, nt = (mut * ht + gamma) / zt;
-    for (int p = 0; p < 4; ++p) {
-        rec[R_DSF + 2 * p] = dSf[p].re;
-        rec[R_DSF + 2 * p + 1] = dSf[p].im;
-        rec[R_DST + 2 * p] = dSt[p].re;
-        rec[R_DST + 2 * p + 1] = dSt[p].im;
-        rec[R_GF + p] = gf[p];
-        rec[R_GT + p] = gt[p];
-        rec[R_LG + p] = lPf * dSf[p].re + lQf * dSf[p].im + lPt * dSt[p].re + lQt * dSt[p].im +
-                        muf * gf[p] + mut * gt[p];
-        rec[R_NG + p] = nf * gf[p] + nt * gt[p];
+    // weights: lamP Re d2S + lamQ Im d2S + 2 mu Re(conj(S) d2S) = wr Re d2S + wi Im d2S
+    const double m2f = 2.0 * muf, m2t = 2.0 * mut;
+    const double wfr = lPf + m2f * Sf.re, wfi = lQf + m2f * Sf.im;
+    const double wtr = lPt + m2t * St.re, wti = lQt + m2t * St.im;
+    const double qf = wfr * a.re + wfi * a.im, rf = wfi * a.re - wfr * a.im;      // of a and j a
+    const double qt = wtr * c.re + wti * c.im, rt = wti * c.re - wtr * c.im;      // of c and j c
+    double H[6] = {neg(p * (qf + qt)), vt * (rf - rt), vf * (rf - rt), 2.0 * (wfr * yff.re - wfi * yff.im), qf + qt,
+                   2.0 * (wtr * ytt.re - wti * ytt.im)};
+    const double bf = muf * rzf, bt = mut * rzt;
+#pragma unroll
+    for (int x = 0, e = 0; x < 3; ++x) {
+        const double fr = m2f * df[2 * x], fi = m2f * df[2 * x + 1], fg = bf * gf[x];
+        const double tr = m2t * dt[2 * x], ti = m2t * dt[2 * x + 1], tg = bt * gt[x];
+#pragma unroll
+        for (int y = x; y < 3; ++y, ++e)
+            H[e] += fr * df[2 * y] + fi * df[2 * y + 1] + fg * gf[y] + tr * dt[2 * y] + ti * dt[2 * y + 1] +
+                    tg * gt[y];
     }
-    rec[R_SF] = Sf.re;
-    rec[R_SF + 1] = Sf.im;
-    rec[R_ST] = St.re;
-    rec[R_ST + 1] = St.im;
+    double2* rec = reinterpret_cast<double2*>(W + L.rec + (size_t)kRec * b);
+#pragma unroll
+    for (int q = 0; q < 3; ++q) {
+        rec[R_H / 2 + q] = make_double2(H[2 * q], H[2 * q + 1]);
+        rec[R_DF / 2 + q] = make_double2(df[2 * q], df[2 * q + 1]);
+        rec[R_DT / 2 + q] = make_double2(dt[2 * q], dt[2 * q + 1]);
+    }
+    rec[R_G / 2] = make_double2(gf[0], gf[1]);
+    rec[R_G / 2 + 1] = make_double2(gf[2], gt[0]);
+    rec[R_G / 2 + 2] = make_double2(gt[1], gt[2]);
+    rec[R_L / 2] = make_double2(lg[0], lg[1]);
+    rec[R_L / 2 + 1] = make_double2(lg[2], ng[0]);
+    rec[R_L / 2 + 2] = make_double2(ng[1], ng[2]);
+    rec[R_S / 2] = make_double2(Sf.re, Sf.im);
+    rec[R_S / 2 + 1] = make_double2(St.re, St.im);
 }
 
 // Solve (L D L^T) v = v in place for the 4-vector-per-bus array v (new order):
@@ -1033,7 +1063,6 @@ opf_kernel(DevNet net, EvalArgs a, const int* islanded, OpfOut o, double tol, in
             W[L.Qg + k] = 0.0;
         }
         __syncthreads();
-        const int ops10[10] = {0, 0, 0, 0, 0, 0, 0, 1, 1, 0};
         int it = 0;
         // evaluate(x) then the convergence quantities; init = first call
         auto evaluate = [&](bool init) {
@@ -1049,50 +1078,56 @@ opf_kernel(DevNet net, EvalArgs a, const int* islanded, OpfOut o, double tol, in
                 eval_branch(net, b, W, L, gamma, init);
             }
             __syncthreads();
-            // per-thread partial reductions: maxg, maxh, maxx, maxz, maxmu, maxLx, maxlam, sumzmu, cost, nonfinite
-            double v[10] = {0.0, -INFINITY, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+            // per-thread partial reductions: max |g|, h, |x|, z, mu, |Lx|, |lam|; sum z mu, cost
+            key_t64 kx[7] = {0, 0, 0, 0, 0, 0, 0};
+            double zmu = 0.0, cost = 0.0;
+            auto top = [&](int q, key_t64 k) { kx[q] = max(kx[q], k); };
             for (int b = tid; b < nbr; b += kThreads) {
                 if (!lv.br(b)) continue;
                 const double zf = W[L.zf + b], zt = W[L.zt + b], mf = W[L.muf + b], mt = W[L.mut + b];
-                v[1] = fmax(v[1], fmax(W[L.hf + b], W[L.ht + b]));
-                v[3] = fmax(v[3], fmax(zf, zt));
-                v[4] = fmax(v[4], fmax(mf, mt));
-                v[7] += zf * mf + zt * mt;
+                top(1, max(pos_key(W[L.hf + b]), pos_key(W[L.ht + b])));
+                top(3, max(abs_key(zf), abs_key(zt)));
+                top(4, max(abs_key(mf), abs_key(mt)));
+                zmu += zf * mf + zt * mt;
             }
             for (int i = tid; i < nb; i += kThreads) {
                 if (!lv.bus(i)) {              // outside the main island: no rows, no bounds, load shed
                     if (init) { W[L.zu + i] = 1.0; W[L.zl + i] = 1.0; W[L.muu + i] = 0.0; W[L.mul + i] = 0.0; }
-                    W[L.gP + i] = 0.0; W[L.gQ + i] = 0.0; W[L.LxVa + i] = 0.0; W[L.LxVm + i] = 0.0;
+                    W[L.rzu + i] = 1.0; W[L.rzl + i] = 1.0;
+                    W[L.gP + i] = 0.0; W[L.gQ + i] = 0.0;
                     W[L.NVa + i] = 0.0; W[L.NVm + i] = 0.0; W[L.DP + i] = 0.0; W[L.DQ + i] = 0.0;
                     W[L.rP + i] = 0.0; W[L.rQ + i] = 0.0;
                     continue;
                 }
                 const double Vm = W[L.Vm + i], Va = W[L.Va + i];
                 const double hu = Vm - net.vmax[i], hl = net.vmin[i] - Vm;
-                double zu, zl, muu, mul;
+                double zu, zl, muu, mul, rzu, rzl;
                 if (init) {
                     zu = fmax(-hu, 1.0); zl = fmax(-hl, 1.0);
-                    muu = gamma / zu; mul = gamma / zl;
+                    rzu = 1.0 / zu; rzl = 1.0 / zl;
+                    muu = gamma * rzu; mul = gamma * rzl;
                     W[L.zu + i] = zu; W[L.zl + i] = zl; W[L.muu + i] = muu; W[L.mul + i] = mul;
                 } else {
                     zu = W[L.zu + i]; zl = W[L.zl + i]; muu = W[L.muu + i]; mul = W[L.mul + i];
+                    rzu = 1.0 / zu; rzl = 1.0 / zl;
                 }
+                W[L.rzu + i] = rzu; W[L.rzl + i] = rzl;
                 const double lP = W[L.lP + i], lQ = W[L.lQ + i];
                 double Sre = Vm * Vm * net.gsh[i], Sim = -Vm * Vm * net.bsh[i];
                 double LxVa = 0.0, LxVm = 2.0 * Vm * (lP * net.gsh[i] - lQ * net.bsh[i]) + muu - mul;
-                double NVa = 0.0, NVm = (muu * hu + gamma) / zu - (mul * hl + gamma) / zl;
+                double NVa = 0.0, NVm = (muu * hu + gamma) * rzu - (mul * hl + gamma) * rzl;
                 for (int e = net.bus_br_ptr[i]; e < net.bus_br_ptr[i + 1]; ++e) {
                     const int code = net.bus_br[e];
                     const int b = code >> 1, side = code & 1;
                     if (!lv.br(b)) continue;
                     const double* rec = W + L.rec + (size_t)kRec * b;
-                    Sre += rec[side ? R_ST : R_SF];
-                    Sim += rec[(side ? R_ST : R_SF) + 1];
-                    const int p0 = 2 * side;
-                    LxVa += rec[R_LG + p0];
-                    LxVm += rec[R_LG + p0 + 1];
-                    NVa += rec[R_NG + p0];
-                    NVm += rec[R_NG + p0 + 1];
+                    const double sg = side ? -1.0 : 1.0;
+                    Sre += rec[R_S + 2 * side];
+                    Sim += rec[R_S + 2 * side + 1];
+                    LxVa += sg * rec[R_L];
+                    LxVm += rec[R_L + 1 + side];
+                    NVa += sg * rec[R_N];
+                    NVm += rec[R_N + 1 + side];
                 }
                 if (i == sc.ref) LxVa += sc.lref;
                 double Pgen = 0.0, Qgen = 0.0, DP = 0.0, DQ = 0.0, rP = 0.0, rQ = 0.0;
@@ -1101,79 +1136,113 @@ opf_kernel(DevNet net, EvalArgs a, const int* islanded, OpfOut o, double tol, in
                     if (!lv.gen(k)) continue;
                     const double Pg = W[L.Pg + k], Qg = W[L.Qg + k];
                     const double h4[4] = {Pg - net.pmax[k], net.pmin[k] - Pg, Qg - net.qmax[k], net.qmin[k] - Qg};
-                    double z4[4], m4[4];
+                    double m4[4], r4[4];
                     for (int q = 0; q < 4; ++q) {
+                        double z;
                         if (init) {
-                            z4[q] = fmax(-h4[q], 1.0);
-                            m4[q] = gamma / z4[q];
-                            W[L.gz + 4 * k + q] = z4[q];
+                            z = fmax(-h4[q], 1.0);
+                            r4[q] = 1.0 / z;
+                            m4[q] = gamma * r4[q];
+                            W[L.gz + 4 * k + q] = z;
                             W[L.gmu + 4 * k + q] = m4[q];
                         } else {
-                            z4[q] = W[L.gz + 4 * k + q];
+                            z = W[L.gz + 4 * k + q];
                             m4[q] = W[L.gmu + 4 * k + q];
+                            r4[q] = 1.0 / z;
                         }
-                        v[1] = fmax(v[1], h4[q]);
-                        v[3] = fmax(v[3], z4[q]);
-                        v[4] = fmax(v[4], m4[q]);
-                        v[7] += z4[q] * m4[q];
+                        W[L.grz + 4 * k + q] = r4[q];
+                        top(1, pos_key(h4[q]));
+                        top(3, abs_key(z));
+                        top(4, abs_key(m4[q]));
+                        zmu += z * m4[q];
                     }
                     const double PgMW = B * Pg;
                     const double LxP = B * (2.0 * net.c2[k] * PgMW + net.c1[k]) - lP + m4[0] - m4[1];
                     const double LxQ = -lQ + m4[2] - m4[3];
-                    const double NP = LxP + (m4[0] * h4[0] + gamma) / z4[0] - (m4[1] * h4[1] + gamma) / z4[1];
-                    const double NQ = LxQ + (m4[2] * h4[2] + gamma) / z4[2] - (m4[3] * h4[3] + gamma) / z4[3];
-                    const double MP = 2.0 * net.c2[k] * B * B + m4[0] / z4[0] + m4[1] / z4[1];
-                    const double MQ = m4[2] / z4[2] + m4[3] / z4[3];
-                    W[L.LxP + k] = LxP; W[L.LxQ + k] = LxQ; W[L.NP + k] = NP; W[L.NQ + k] = NQ;
-                    W[L.MP + k] = MP; W[L.MQ + k] = MQ;
-                    DP += 1.0 / MP;
-                    DQ += 1.0 / MQ;
-                    rP += NP / MP;
-                    rQ += NQ / MQ;
+                    const double NP = LxP + (m4[0] * h4[0] + gamma) * r4[0] - (m4[1] * h4[1] + gamma) * r4[1];
+                    const double NQ = LxQ + (m4[2] * h4[2] + gamma) * r4[2] - (m4[3] * h4[3] + gamma) * r4[3];
+                    const double rMP = 1.0 / (2.0 * net.c2[k] * B * B + m4[0] * r4[0] + m4[1] * r4[1]);
+                    const double rMQ = 1.0 / (m4[2] * r4[2] + m4[3] * r4[3]);
+                    W[L.NP + k] = NP; W[L.NQ + k] = NQ;
+                    W[L.MP + k] = rMP; W[L.MQ + k] = rMQ;
+                    DP += rMP;
+                    DQ += rMQ;
+                    rP += NP * rMP;
+                    rQ += NQ * rMQ;
                     Pgen += Pg;
                     Qgen += Qg;
-                    v[2] = fmax(v[2], fmax(fabs(Pg), fabs(Qg)));
-                    v[5] = fmax(v[5], fmax(fabs(LxP), fabs(LxQ)));
-                    v[8] += net.c2[k] * PgMW * PgMW + net.c1[k] * PgMW + net.c0[k];
+                    top(2, max(abs_key(Pg), abs_key(Qg)));
+                    top(5, max(abs_key(LxP), abs_key(LxQ)));
+                    cost += net.c2[k] * PgMW * PgMW + net.c1[k] * PgMW + net.c0[k];
                 }
                 NVa += LxVa;
                 NVm += LxVm;
                 const double gP = Sre - Pgen + Pd[i], gQ = Sim - Qgen + Qd[i];
                 W[L.gP + i] = gP; W[L.gQ + i] = gQ;
-                W[L.LxVa + i] = LxVa; W[L.LxVm + i] = LxVm; W[L.NVa + i] = NVa; W[L.NVm + i] = NVm;
+                W[L.NVa + i] = NVa; W[L.NVm + i] = NVm;
                 W[L.DP + i] = DP; W[L.DQ + i] = DQ; W[L.rP + i] = rP; W[L.rQ + i] = rQ;
-                v[0] = fmax(v[0], fmax(fabs(gP), fabs(gQ)));
-                v[1] = fmax(v[1], fmax(hu, hl));
-                v[2] = fmax(v[2], fmax(fabs(Va), fabs(Vm)));
-                v[3] = fmax(v[3], fmax(zu, zl));
-                v[4] = fmax(v[4], fmax(muu, mul));
-                v[5] = fmax(v[5], fmax(fabs(LxVa), fabs(LxVm)));
-                v[6] = fmax(v[6], fmax(fabs(lP), fabs(lQ)));
-                v[7] += zu * muu + zl * mul;
-                if (!isfinite(gP) || !isfinite(gQ) || !isfinite(NVa) || !isfinite(NVm)) v[9] = 1.0;
+                top(0, max(abs_key(gP), abs_key(gQ)));
+                if (non_finite(NVa) || non_finite(NVm)) top(0, 0x7ff0000000000000ull);
+                top(1, max(pos_key(hu), pos_key(hl)));
+                top(2, max(abs_key(Va), abs_key(Vm)));
+                top(3, max(abs_key(zu), abs_key(zl)));
+                top(4, max(abs_key(muu), abs_key(mul)));
+                top(5, max(abs_key(LxVa), abs_key(LxVm)));
+                top(6, max(abs_key(lP), abs_key(lQ)));
+                zmu += zu * muu + zl * mul;
             }
-            if (tid == 0) v[6] = fmax(v[6], fabs(sc.lref));
-            block_reduce<10>(rb, v, ops10, sc.red);
-            if (tid == 0) {
-                const double maxg = sc.red[0], maxh = sc.red[1], maxx = sc.red[2], maxz = sc.red[3];
-                const double maxmu = sc.red[4], maxLx = sc.red[5], maxlam = sc.red[6], zmu = sc.red[7];
-                sc.f = sc.red[8];
-                if (init) sc.f_prev = sc.f;
-                const double feas = fmax(maxg, maxh) / (1.0 + fmax(maxx, maxz));
-                const double grad = maxLx / (1.0 + fmax(maxlam, maxmu));
-                const double comp = zmu / (1.0 + maxx);
-                const double cost = fabs(sc.f - sc.f_prev) / (1.0 + fabs(sc.f_prev));
-                if (sc.red[9] != 0.0 || !isfinite(sc.f) || !isfinite(feas) || !isfinite(grad) || !isfinite(comp))
-                    sc.fail = 1;
-                sc.conv = (feas < tol && grad < tol && comp < tol && cost < tol) ? 1 : 0;
-                // One step keeps at least the fraction 1 - xi = 5e-5 of every z and of every mu, so
-                // the complementarity loses less than 2^29 per iteration.  A point further than
-                // 30 bits per remaining iteration (and 100 more) above the tolerance cannot
-                // converge any more: on an infeasible scenario the multipliers grow by decades per
-                // iteration, and the iterations saved are those whose Newton systems need the dense
-                // backstop (and may overflow).
-                if (sc.red[7] > 0.0 && isfinite(comp))
-                    sc.lost = ilogb(comp) > ilogb(tol) + 100 + kLossBits * (max_it - it) ? 1 : 0;
+            if (tid == 0) top(6, abs_key(sc.lref));
+#pragma unroll
+            for (int q = 0; q < 7; ++q) kx[q] = warp_max_key(kx[q]);
+            for (int off = 16; off; off >>= 1) {
+                zmu += __shfl_xor_sync(0xffffffffu, zmu, off);
+                cost += __shfl_xor_sync(0xffffffffu, cost, off);
+            }
+            if ((tid & 31) == 0) {
+#pragma unroll
+                for (int q = 0; q < 7; ++q) rb.v[q][tid >> 5] = key_value(kx[q]);
+                rb.v[7][tid >> 5] = zmu;
+                rb.v[8][tid >> 5] = cost;
+            }
+            __syncthreads();
+            if (tid < 32) {
+                // every lane takes the totals; lanes 0..3 divide for one stopping condition each
+                key_t64 mx[7];
+#pragma unroll
+                for (int q = 0; q < 7; ++q) {
+                    mx[q] = 0;
+                    for (int w = 0; w < kWarps; ++w) mx[q] = max(mx[q], abs_key(rb.v[q][w]));
+                }
+                double zm = rb.v[7][0], f = rb.v[8][0];
+                for (int w = 1; w < kWarps; ++w) {
+                    zm += rb.v[7][w];
+                    f += rb.v[8][w];
+                }
+                const double fp = init ? f : sc.f_prev;
+                // feasibility (the largest |g| is at least 0, so only a positive h can decide it),
+                // gradient, complementarity, cost
+                const double num = tid == 0 ? key_value(max(mx[0], mx[1])) : tid == 1 ? key_value(mx[5])
+                                 : tid == 2 ? zm : fabs(f - fp);
+                const double den = 1.0 + (tid == 0 ? key_value(max(mx[2], mx[3]))
+                                        : tid == 1 ? key_value(max(mx[6], mx[4]))
+                                        : tid == 2 ? key_value(mx[2]) : fabs(fp));
+                const double cnd = num / den;
+                const unsigned wild = __ballot_sync(0xffffffffu, non_finite(cnd) || non_finite(f)) & 0xfu;
+                const unsigned met = __ballot_sync(0xffffffffu, cnd < tol) & 0xfu;
+                if (tid == 2) {
+                    sc.f = f;
+                    if (init) sc.f_prev = f;
+                    if (wild) sc.fail = 1;
+                    sc.conv = met == 0xfu ? 1 : 0;
+                    // One step keeps at least the fraction 1 - xi = 5e-5 of every z and of every mu, so
+                    // the complementarity loses less than 2^29 per iteration.  A point further than
+                    // 30 bits per remaining iteration (and 100 more) above the tolerance cannot
+                    // converge any more: on an infeasible scenario the multipliers grow by decades per
+                    // iteration, and the iterations saved are those whose Newton systems need the dense
+                    // backstop (and may overflow).
+                    if (zm > 0.0 && !non_finite(cnd))
+                        sc.lost = ilogb(cnd) > ilogb(tol) + 100 + kLossBits * (max_it - it) ? 1 : 0;
+                }
             }
             __syncthreads();
         };
@@ -1192,21 +1261,23 @@ opf_kernel(DevNet net, EvalArgs a, const int* islanded, OpfOut o, double tol, in
                     const double Vm = W[L.Vm + i];
                     double J[2][2] = {{0.0, 2.0 * net.gsh[i] * Vm}, {0.0, -2.0 * net.bsh[i] * Vm}};
                     blk[5] = 2.0 * (W[L.lP + i] * net.gsh[i] - W[L.lQ + i] * net.bsh[i]) +
-                             W[L.muu + i] / W[L.zu + i] + W[L.mul + i] / W[L.zl + i];
+                             W[L.muu + i] * W[L.rzu + i] + W[L.mul + i] * W[L.rzl + i];
                     for (int e = net.bus_br_ptr[i]; e < net.bus_br_ptr[i + 1]; ++e) {
                         const int code = net.bus_br[e];
                         const int b = code >> 1, side = code & 1;
                         if (!lv.br(b)) continue;
                         const double* rec = W + L.rec + (size_t)kRec * b;
-                        const int p0 = 2 * side;
-                        const double* dS = rec + (side ? R_DST : R_DSF);
-                        for (int r = 0; r < 2; ++r)
-                            for (int c = 0; c < 2; ++c) blk[4 * r + c] += rec[R_H + hidx(p0 + r, p0 + c)];
-                        for (int c = 0; c < 2; ++c) {
-                            J[0][c] += dS[2 * (p0 + c)];
-                            J[1][c] += dS[2 * (p0 + c) + 1];
-                        }
+                        const double sg = side ? -1.0 : 1.0;
+                        const double* dS = rec + (side ? R_DT : R_DF);
+                        blk[0] += rec[R_H];
+                        blk[1] += sg * rec[R_H + 1 + side];
+                        blk[5] += rec[side ? R_H + 5 : R_H + 3];
+                        J[0][0] += sg * dS[0];
+                        J[1][0] += sg * dS[1];
+                        J[0][1] += dS[2 + 2 * side];
+                        J[1][1] += dS[3 + 2 * side];
                     }
+                    blk[4] = blk[1];
                     for (int q = 0; q < 2; ++q)
                         for (int r = 0; r < 2; ++r) {
                             blk[4 * r + 2 + q] = J[q][r];
@@ -1241,16 +1312,14 @@ opf_kernel(DevNet net, EvalArgs a, const int* islanded, OpfOut o, double tol, in
                         if (!lv.br(b)) continue;
                         const double* rec = W + L.rec + (size_t)kRec * b;
                         const bool flip = (net.f[b] != Rb);     // stored block is (t row, f col)
-                        double K[16];
-                        for (int r = 0; r < 4; ++r)
-                            for (int c = 0; c < 4; ++c) {
-                                double v;
-                                if (r < 2 && c < 2) v = rec[R_H + hidx(r, 2 + c)];
-                                else if (r < 2) v = rec[R_DST + 2 * r + (c - 2)];          // J(t,f)^T
-                                else if (c < 2) v = rec[R_DSF + 2 * (2 + c) + (r - 2)];    // J(f,t)
-                                else v = 0.0;
-                                K[4 * r + c] = v;
-                            }
+                        const double* H = rec + R_H;
+                        const double* DF = rec + R_DF;
+                        const double* DT = rec + R_DT;
+                        // rows (theta_f, Vm_f, lamP_f, lamQ_f), columns the same of t
+                        const double K[16] = {neg(H[0]), H[2], DT[0], DT[1],
+                                              neg(H[1]), H[4], DT[2], DT[3],
+                                              neg(DF[0]), DF[4], 0.0, 0.0,
+                                              neg(DF[1]), DF[5], 0.0, 0.0};
                         for (int r = 0; r < 4; ++r)
                             for (int c = 0; c < 4; ++c) blk[4 * r + c] += flip ? K[4 * c + r] : K[4 * r + c];
                     }
@@ -1375,48 +1444,42 @@ opf_kernel(DevNet net, EvalArgs a, const int* islanded, OpfOut o, double tol, in
                 }
             }
             // ---------------- recover the eliminated steps, dz, dmu, ratios ----------------
-            double rp = INFINITY, rd = INFINITY, bad = 0.0;
+            // Step lengths: xi over the largest -dz / z and -dmu / mu of all rows; the first is a
+            // product with the stored 1 / z.
+            key_t64 kp = 0, kd = 0;
+            bool bad = false;
+            auto row = [&](double rz, double m, double dz, int odz, int odm) {
+                const double dm = (gamma - m * dz) * rz - m;
+                W[odz] = dz;
+                W[odm] = dm;
+                kp = max(kp, pos_key(neg(dz) * rz));
+                if (__double2hiint(dm) < 0) kd = max(kd, pos_key(neg(dm) / m));
+                bad = bad || non_finite(dz) || non_finite(dm);
+            };
             for (int k = tid; k < ng; k += kThreads) {
                 if (!lv.gen(k)) continue;
                 const int jn = net.iperm[net.gbus[k]];
-                const double dlP = W[L.x + 4 * jn + 2], dlQ = W[L.x + 4 * jn + 3];
-                const double dPg = (-W[L.NP + k] + dlP) / W[L.MP + k];
-                const double dQg = (-W[L.NQ + k] + dlQ) / W[L.MQ + k];
+                const double dPg = (W[L.x + 4 * jn + 2] - W[L.NP + k]) * W[L.MP + k];
+                const double dQg = (W[L.x + 4 * jn + 3] - W[L.NQ + k]) * W[L.MQ + k];
                 W[L.dPg + k] = dPg;
                 W[L.dQg + k] = dQg;
                 const double Pg = W[L.Pg + k], Qg = W[L.Qg + k];
                 const double h4[4] = {Pg - net.pmax[k], net.pmin[k] - Pg, Qg - net.qmax[k], net.qmin[k] - Qg};
-                const double dh4[4] = {dPg, -dPg, dQg, -dQg};
-                for (int q = 0; q < 4; ++q) {
-                    const double z = W[L.gz + 4 * k + q], m = W[L.gmu + 4 * k + q];
-                    const double dz = -h4[q] - z - dh4[q];
-                    const double dm = -m + (gamma - m * dz) / z;
-                    W[L.gdz + 4 * k + q] = dz;
-                    W[L.gdmu + 4 * k + q] = dm;
-                    if (dz < 0.0) rp = fmin(rp, -z / dz);
-                    if (dm < 0.0) rd = fmin(rd, -m / dm);
-                    if (!isfinite(dz) || !isfinite(dm)) bad = 1.0;
-                }
+                const double dh4[4] = {dPg, neg(dPg), dQg, neg(dQg)};
+                for (int q = 0; q < 4; ++q)
+                    row(W[L.grz + 4 * k + q], W[L.gmu + 4 * k + q], -h4[q] - W[L.gz + 4 * k + q] - dh4[q],
+                        L.gdz + 4 * k + q, L.gdmu + 4 * k + q);
             }
             for (int b = tid; b < nbr; b += kThreads) {
                 if (!lv.br(b)) continue;
-                const double* rec = W + L.rec + (size_t)kRec * b;
-                const int fn = net.iperm[net.f[b]], tn = net.iperm[net.t[b]];
-                const double dx[4] = {W[L.x + 4 * fn], W[L.x + 4 * fn + 1], W[L.x + 4 * tn], W[L.x + 4 * tn + 1]};
-                double gdf = 0.0, gdt = 0.0;
-                for (int p = 0; p < 4; ++p) {
-                    gdf += rec[R_GF + p] * dx[p];
-                    gdt += rec[R_GT + p] * dx[p];
-                }
-                const double zf = W[L.zf + b], zt = W[L.zt + b], mf = W[L.muf + b], mt = W[L.mut + b];
-                const double dzf = -W[L.hf + b] - zf - gdf, dzt = -W[L.ht + b] - zt - gdt;
-                const double dmf = -mf + (gamma - mf * dzf) / zf, dmt = -mt + (gamma - mt * dzt) / zt;
-                W[L.dzf + b] = dzf; W[L.dzt + b] = dzt; W[L.dmuf + b] = dmf; W[L.dmut + b] = dmt;
-                if (dzf < 0.0) rp = fmin(rp, -zf / dzf);
-                if (dzt < 0.0) rp = fmin(rp, -zt / dzt);
-                if (dmf < 0.0) rd = fmin(rd, -mf / dmf);
-                if (dmt < 0.0) rd = fmin(rd, -mt / dmt);
-                if (!isfinite(dzf) || !isfinite(dzt) || !isfinite(dmf) || !isfinite(dmt)) bad = 1.0;
+                const double* G = W + L.rec + (size_t)kRec * b + R_G;
+                const double* xf = W + L.x + 4 * net.iperm[net.f[b]];
+                const double* xt = W + L.x + 4 * net.iperm[net.t[b]];
+                const double dth = xf[0] - xt[0], df = xf[1], dt = xt[1];
+                row(W[L.rzf + b], W[L.muf + b], -W[L.hf + b] - W[L.zf + b] - (G[0] * dth + G[1] * df + G[2] * dt),
+                    L.dzf + b, L.dmuf + b);
+                row(W[L.rzt + b], W[L.mut + b], -W[L.ht + b] - W[L.zt + b] - (G[3] * dth + G[4] * df + G[5] * dt),
+                    L.dzt + b, L.dmut + b);
             }
             for (int i = tid; i < nb; i += kThreads) {
                 if (!lv.bus(i)) continue;
@@ -1424,44 +1487,47 @@ opf_kernel(DevNet net, EvalArgs a, const int* islanded, OpfOut o, double tol, in
                 const double dVm = W[L.x + 4 * jn + 1];
                 const double Vm = W[L.Vm + i];
                 const double hu = Vm - net.vmax[i], hl = net.vmin[i] - Vm;
-                const double zu = W[L.zu + i], zl = W[L.zl + i], mu_ = W[L.muu + i], ml = W[L.mul + i];
-                const double dzu = -hu - zu - dVm, dzl = -hl - zl + dVm;
-                const double dmu = -mu_ + (gamma - mu_ * dzu) / zu, dml = -ml + (gamma - ml * dzl) / zl;
-                W[L.dzu + i] = dzu; W[L.dzl + i] = dzl; W[L.dmuu + i] = dmu; W[L.dmul + i] = dml;
-                if (dzu < 0.0) rp = fmin(rp, -zu / dzu);
-                if (dzl < 0.0) rp = fmin(rp, -zl / dzl);
-                if (dmu < 0.0) rd = fmin(rd, -mu_ / dmu);
-                if (dml < 0.0) rd = fmin(rd, -ml / dml);
-                for (int r = 0; r < 4; ++r)
-                    if (!isfinite(W[L.x + 4 * jn + r])) bad = 1.0;
+                row(W[L.rzu + i], W[L.muu + i], -hu - W[L.zu + i] - dVm, L.dzu + i, L.dmuu + i);
+                row(W[L.rzl + i], W[L.mul + i], -hl - W[L.zl + i] + dVm, L.dzl + i, L.dmul + i);
+                for (int r = 0; r < 4; ++r) bad = bad || non_finite(W[L.x + 4 * jn + r]);
             }
-            if (tid == 0) {
+            if (tid == kThreads - 1) {         // a warp with few rows of its own above
                 // multiplier step of the reference-angle row from its Newton row
                 const int i = sc.ref;
-                double row = 0.0;
+                double sum = 0.0;
                 for (int e = net.bus_br_ptr[i]; e < net.bus_br_ptr[i + 1]; ++e) {
                     const int code = net.bus_br[e];
                     const int b = code >> 1, side = code & 1;
                     if (!lv.br(b)) continue;
                     const double* rec = W + L.rec + (size_t)kRec * b;
-                    const int fn = net.iperm[net.f[b]], tn = net.iperm[net.t[b]];
-                    const double dx[4] = {W[L.x + 4 * fn], W[L.x + 4 * fn + 1], W[L.x + 4 * tn], W[L.x + 4 * tn + 1]};
-                    const int p = 2 * side;
-                    for (int q = 0; q < 4; ++q) row += rec[R_H + hidx(p, q)] * dx[q];
-                    row += rec[R_DSF + 2 * p] * W[L.x + 4 * fn + 2] + rec[R_DSF + 2 * p + 1] * W[L.x + 4 * fn + 3];
-                    row += rec[R_DST + 2 * p] * W[L.x + 4 * tn + 2] + rec[R_DST + 2 * p + 1] * W[L.x + 4 * tn + 3];
+                    const double* xf = W + L.x + 4 * net.iperm[net.f[b]];
+                    const double* xt = W + L.x + 4 * net.iperm[net.t[b]];
+                    const double th = rec[R_H] * (xf[0] - xt[0]) + rec[R_H + 1] * xf[1] + rec[R_H + 2] * xt[1] +
+                                      rec[R_DF] * xf[2] + rec[R_DF + 1] * xf[3] + rec[R_DT] * xt[2] +
+                                      rec[R_DT + 1] * xt[3];
+                    sum += side ? neg(th) : th;
                 }
-                sc.dlref = -W[L.NVa + i] - row;
+                sc.dlref = -W[L.NVa + i] - sum;
+                bad = bad || non_finite(sc.dlref);
             }
-            {
-                double v3[3] = {rp, rd, bad};
-                const int ops3[3] = {2, 2, 0};
-                block_reduce<3>(rb, v3, ops3, sc.red);
+            kp = warp_max_key(kp);
+            kd = warp_max_key(kd);
+            bad = __any_sync(0xffffffffu, bad);
+            if ((tid & 31) == 0) {
+                rb.v[0][tid >> 5] = key_value(kp);
+                rb.v[1][tid >> 5] = key_value(kd);
+                rb.v[2][tid >> 5] = bad ? 1.0 : 0.0;
             }
-            if (tid == 0) {
-                sc.ap = fmin(kXi * sc.red[0], 1.0);
-                sc.ad = fmin(kXi * sc.red[1], 1.0);
-                if (sc.red[2] != 0.0 || !isfinite(sc.dlref)) sc.fail = 1;
+            __syncthreads();
+            if (tid < 2) {
+                key_t64 k = 0;
+                for (int w = 0; w < kWarps; ++w) {
+                    k = max(k, abs_key(rb.v[tid][w]));
+                    if (rb.v[2][w] != 0.0) sc.fail = 1;
+                }
+                const double al = fmin(kXi / key_value(k), 1.0);   // no row decreases: 1
+                if (tid == 0) sc.ap = al;
+                else sc.ad = al;
             }
             __syncthreads();
             if (sc.fail) break;
