@@ -481,6 +481,7 @@ cs_status cs_load_network(cs_ctx* ctx, const cs_network_desc* d, int32_t* net_id
     std::vector<int> f(d->f, d->f + nbr), t(d->t, d->t + nbr);
     std::string msg = symbolic_analysis(nb, f, t, d->ref_bus, net->sym);
     if (!msg.empty()) return fail(ctx, CS_E_ARG, msg);
+    level_shares(opf_groups(), net->sym);
     const Symbolic& S = net->sym;
     const double B = d->base_mva;
     // per-unit conversion and branch two-port admittances
@@ -553,7 +554,9 @@ cs_status cs_load_network(cs_ctx* ctx, const cs_network_desc* d, int32_t* net_id
            o_Lc = P.add(S.Lcol), o_Lrp = P.add(S.Lrowptr), o_Lrc = P.add(S.Lrowcol), o_Lrb = P.add(S.Lrowblk),
            o_lp = P.add(S.lev_ptr), o_lc = P.add(S.lev_col), o_tp = P.add(S.tgt_ptr), o_tg = P.add(S.tgt),
            o_up = P.add(S.upd_ptr), o_ua = P.add(S.upd_a), o_ub = P.add(S.upd_b), o_bbrp = P.add(S.blk_br_ptr),
-           o_bbr = P.add(S.blk_br);
+           o_bbr = P.add(S.blk_br), o_ap = P.add(S.adj_ptr), o_ac = P.add(S.adj_col), o_ab = P.add(S.adj_blk),
+           o_rnp = P.add(S.rn_ptr), o_rnf = P.add(S.rn_first), o_rne = P.add(S.rn_end), o_sha = P.add(S.sh_a),
+           o_shb = P.add(S.sh_b), o_ofp = P.add(S.off_ptr), o_off = P.add(S.off);
     if (ctx->opt.hbm_budget > 0) {                    // admission by device footprint
         const int64_t ne = (int64_t)nbr + ng;
         const size_t add = P.host.size() + (size_t)nlev * (size_t)(ne + ne * (ne - 1) / 2);
@@ -586,6 +589,9 @@ cs_status cs_load_network(cs_ctx* ctx, const cs_network_desc* d, int32_t* net_id
     dn.nlevels = S.nlevels; dn.lev_ptr = P_(int, o_lp); dn.lev_col = P_(int, o_lc); dn.tgt_ptr = P_(int, o_tp);
     dn.tgt = P_(int, o_tg); dn.upd_ptr = P_(int, o_up); dn.upd_a = P_(int, o_ua); dn.upd_b = P_(int, o_ub);
     dn.blk_br_ptr = P_(int, o_bbrp); dn.blk_br = P_(int, o_bbr);
+    dn.adj_ptr = P_(int, o_ap); dn.adj_col = P_(int, o_ac); dn.adj_blk = P_(int, o_ab);
+    dn.rn_ptr = P_(int, o_rnp); dn.rn_first = P_(int, o_rnf); dn.rn_end = P_(int, o_rne);
+    dn.sh_a = P_(int, o_sha); dn.sh_b = P_(int, o_shb); dn.off_ptr = P_(int, o_ofp); dn.off = P_(int4, o_off);
 #undef P_
     // severity tables, one per level, 255 = not evaluated
     const int64_t nE = nbr + ng;

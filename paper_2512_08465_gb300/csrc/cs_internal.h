@@ -97,6 +97,16 @@ struct DevNet {
     const int* upd_b;               // block (j,k)
     const int* blk_br_ptr;          // [nL + 1] branches whose off-diagonal pair is block q
     const int* blk_br;
+    const int* rn_ptr;              // [nlevels * opf_groups() + 1] the block updates of each level in equal
+    const int* rn_first;            // shares (symbolic.h: level_shares)
+    const int* rn_end;
+    const int* sh_a;
+    const int* sh_b;
+    const int* off_ptr;             // [nlevels + 1] the off-diagonal blocks of each level
+    const int4* off;
+    const int* adj_ptr;             // [nb + 1] per row (new index) its blocks that hold a branch:
+    const int* adj_col;             // column of the block
+    const int* adj_blk;             // 2 * block id, + 1 if the row reads the block transposed
 };
 
 // scenario masks: up to two outaged elements
@@ -160,6 +170,7 @@ cudaError_t launch_opf(const DevNet& net, const EvalArgs& a, const int* islanded
                        double tol, int max_it, double* scratch, size_t scratch_per_cta, int grid,
                        int* counter, cudaStream_t s);
 size_t opf_scratch_doubles(const DevNet& net);
+int opf_groups();            // groups of 16 threads that share the updates of one level
 int opf_ctas_per_sm();       // resident OPF CTAs per SM the kernel is built for
 // Small-signal screen.  counters: 5 work counters (zeroed by the caller).
 // abuf, hbuf, a64, cand (mixed form, NULL otherwise): a.n * dyn_abuf_stride(net)

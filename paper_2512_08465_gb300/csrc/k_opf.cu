@@ -26,7 +26,7 @@
 //  * that matrix is factorised as a block LDL^T on ONE symbolic analysis per
 //    network (minimum-degree order, elimination tree, fill pattern and
 //    left-looking update lists, built on the host at load time), with the
-//    4x4 pivot blocks inverted by Gauss-Jordan with partial pivoting.  Columns
+//    4x4 pivot blocks inverted by LU with partial pivoting.  Columns
 //    of one elimination-tree level are independent, so a level is one
 //    parallel step of the CTA (16 threads per target block).  The narrow
 //    upper levels leave most threads at barriers, so CTAs are small (128
@@ -59,6 +59,11 @@ namespace {
 constexpr int kThreads = CS_OPF_THREADS;   // threads per scenario CTA
 constexpr int kCtasPerSm = CS_OPF_CTAS;    // resident CTAs per SM the register budget is sized for
 constexpr int kWarps = kThreads / 32;
+constexpr int kGroups = kThreads / 16;     // groups of 16 threads, one thread per entry of a 4x4 block
+#ifndef CS_OPF_BATCH
+#define CS_OPF_BATCH 4
+#endif
+constexpr int kBatch = CS_OPF_BATCH;       // block updates whose loads are in flight together
 constexpr int kRec = 34;     // doubles per branch record
 constexpr double kXi = 0.99995;
 constexpr double kSigma = 0.1;
@@ -201,64 +206,130 @@ __device__ void block_reduce(RedBuf& rb, double (&val)[K], const int (&ops)[K], 
 // then symmetrisation of the result.  (Near the end of the interior-point
 // iteration some pivot blocks are nearly singular; the LU-based inverse keeps
 // the error low-rank, which the iterative refinement removes, where a
-// Gauss-Jordan inverse did not.)  Four lanes of one warp (q = 0..3, aligned
-// to a multiple of 4) take one pivot: each repeats the factorisation (one
-// instruction stream, so the FP64 pipe pays for it once) and solves for column
-// q.  Returns false, on all four lanes, if a pivot is exactly zero or not
-// finite.
-__device__ bool inv4(const double* A, double* Ainv, int q) {
-    const unsigned grp = 0xFu << (threadIdx.x & 28);
+// Gauss-Jordan inverse did not.)  Two forms of the same steps:
+//  * inv4_wide, four lanes a pivot, for levels with many columns: each lane repeats the
+//    factorisation and solves for column q; ~77 FP64 instructions for eight pivots per warp;
+//  * inv4, sixteen lanes a pivot, one entry each (lane e = 4 r + c: a = A(r, c), the result
+//    Ainv(r, c)), for the top of the tree, where every level waits for one pivot's chain of
+//    dependent FP64 instructions: ~41 of them.
+// ok becomes false, on all lanes of the group (mask grp), if a pivot is exactly zero or not finite.
+__device__ void inv4_wide(const double* A, double* Ainv, int q, unsigned grp, bool& ok) {
     double a[4][4], dinv[4];
     int piv[4] = {0, 1, 2, 3};
-    for (int r = 0; r < 4; ++r)                  // symmetric part of the updated pivot
-        for (int c = 0; c < 4; ++c) a[r][c] = 0.5 * (A[4 * r + c] + A[4 * c + r]);
-    bool ok = true;
-    for (int c = 0; c < 4 && ok; ++c) {
-        int p = c;
-        double best = fabs(a[c][c]);
-        for (int r = c + 1; r < 4; ++r)
-            if (fabs(a[r][c]) > best) { best = fabs(a[r][c]); p = r; }
-        if (!(best > 0.0) || !isfinite(best)) { ok = false; break; }
-        if (p != c) {
-            for (int k = 0; k < 4; ++k) { double t = a[c][k]; a[c][k] = a[p][k]; a[p][k] = t; }
-            int t = piv[c]; piv[c] = piv[p]; piv[p] = t;
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+        a[r][r] = A[5 * r];
+#pragma unroll
+        for (int c = 0; c < r; ++c) a[c][r] = a[r][c] = 0.5 * (A[4 * r + c] + A[4 * c + r]);
+    }
+    ok = true;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        int p = k;
+        key_t64 best = abs_key(a[k][k]);
+        if (best > 0x7ff0000000000000ull) ok = false;   // NaN on the diagonal
+#pragma unroll
+        for (int r = k + 1; r < 4; ++r) {
+            const key_t64 v = abs_key(a[r][k]);
+            if (v > best && v <= 0x7ff0000000000000ull) { best = v; p = r; }
         }
-        dinv[c] = 1.0 / a[c][c];                  // one division per pivot
-        for (int r = c + 1; r < 4; ++r) {
-            a[r][c] *= dinv[c];
-            const double m = a[r][c];
-            for (int k = c + 1; k < 4; ++k) a[r][k] -= m * a[c][k];
+        if (best == 0ull || best >= 0x7ff0000000000000ull) ok = false;
+#pragma unroll
+        for (int r = k + 1; r < 4; ++r)
+            if (p == r) {                               // rows k and p trade places
+#pragma unroll
+                for (int c = 0; c < 4; ++c) { const double t = a[k][c]; a[k][c] = a[r][c]; a[r][c] = t; }
+                const int t = piv[k]; piv[k] = piv[r]; piv[r] = t;
+            }
+        dinv[k] = 1.0 / a[k][k];
+#pragma unroll
+        for (int r = k + 1; r < 4; ++r) {
+            a[r][k] *= dinv[k];
+#pragma unroll
+            for (int c = k + 1; c < 4; ++c) a[r][c] -= a[r][k] * a[k][c];
         }
     }
-    // the group reads A above before any lane of it writes the inverse (A and Ainv
-    // are different arrays, but the symmetrisation below reads what others wrote)
     double y[4];
-    if (ok) {
-        for (int i = 0; i < 4; ++i) {
-            double v = (piv[i] == q) ? 1.0 : 0.0;
-            for (int k = 0; k < i; ++k) v -= a[i][k] * y[k];
-            y[i] = v;
-        }
-        for (int i = 3; i >= 0; --i) {
-            double v = y[i];
-            for (int k = i + 1; k < 4; ++k) v -= a[i][k] * y[k];
-            y[i] = v * dinv[i];
-        }
-        for (int i = 0; i < 4; ++i) Ainv[4 * i + q] = y[i];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        double v = (piv[i] == q) ? 1.0 : 0.0;
+#pragma unroll
+        for (int k = 0; k < i; ++k) v -= a[i][k] * y[k];
+        y[i] = v;
     }
-    __syncwarp(grp);
+#pragma unroll
+    for (int i = 3; i >= 0; --i) {
+        double v = y[i];
+#pragma unroll
+        for (int k = i + 1; k < 4; ++k) v -= a[i][k] * y[k];
+        y[i] = v * dinv[i];
+    }
+    // symmetrised below (see inv4): entry (i, q) meets entry (q, i), which lane i holds as its y[q]
+    const int base = threadIdx.x & 28;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        double t = 0.0;
+#pragma unroll
+        for (int s = 0; s < 4; ++s) {                   // lane q sends y[s] to the lane that wants it
+            const double v = __shfl_sync(grp, y[s], base + i);
+            if (s == q) t = v;
+        }
+        Ainv[4 * i + q] = 0.5 * (y[i] + t);
+    }
+}
+
+__device__ double inv4(double a, unsigned grp, bool& ok) {
+    const int lane = threadIdx.x & 31, e = lane & 15, base = lane & 16, r = e >> 2, c = e & 3;
+    a = 0.5 * (a + __shfl_sync(grp, a, base + 4 * c + r));
+    double dinv[4];
+    int perm = 0x3210;                                  // original row of row i in bits 4 i .. 4 i + 3
+    ok = true;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        double col[4];
+#pragma unroll
+        for (int i = k; i < 4; ++i) col[i] = __shfl_sync(grp, a, base + 4 * i + k);
+        int p = k;
+        key_t64 best = abs_key(col[k]);
+        if (best > 0x7ff0000000000000ull) ok = false;   // NaN on the diagonal
+#pragma unroll
+        for (int i = k + 1; i < 4; ++i) {
+            const key_t64 v = abs_key(col[i]);
+            if (v > best && v <= 0x7ff0000000000000ull) { best = v; p = i; }
+        }
+        if (best == 0ull || best >= 0x7ff0000000000000ull) ok = false;
+        const double piv = p == k ? col[k] : p == k + 1 ? col[k < 3 ? k + 1 : 3] : p == 2 ? col[2] : col[3];
+        const int src = r == k ? p : r == p ? k : r;    // rows k and p trade places
+        a = __shfl_sync(grp, a, base + 4 * src + c);
+        const int pk = (perm >> (4 * k)) & 15, pp = (perm >> (4 * p)) & 15;
+        perm = (perm & ~(15 << (4 * k)) & ~(15 << (4 * p))) | (pp << (4 * k));
+        if (p != k) perm |= pk << (4 * p);
+        dinv[k] = 1.0 / piv;
+        double mine = col[k];                           // column k of this lane's row after the exchange
+#pragma unroll
+        for (int i = k; i < 4; ++i)
+            if (src == i) mine = col[i];
+        const double m = mine * dinv[k];
+        const double u = __shfl_sync(grp, a, base + 4 * k + c);
+        if (r > k) a = (c == k) ? m : (c > k ? a - m * u : a);
+    }
+    double y = ((perm >> (4 * r)) & 15) == c ? 1.0 : 0.0;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        const double yk = __shfl_sync(grp, y, base + 4 * k + c), l = __shfl_sync(grp, a, base + 4 * r + k);
+        if (r > k) y -= l * yk;
+    }
+#pragma unroll
+    for (int k = 3; k >= 0; --k) {
+        const double xk = __shfl_sync(grp, y, base + 4 * k + c) * dinv[k], u = __shfl_sync(grp, a, base + 4 * r + k);
+        if (r == k) y = xk;
+        if (r < k) y -= u * xk;
+    }
     // Symmetrise.  Only the lower blocks are stored and updated with L(i,k) U(j,k)^T,
     // which assumes a symmetric pivot inverse; an LU-based inverse of a nearly singular
     // symmetric block is far from symmetric in rounding, and the factorisation would
     // then not be a consistent L D L^T (refinement stalls).
-    double t[4];
-    if (ok)
-        for (int i = 0; i < 4; ++i) t[i] = Ainv[4 * q + i];   // row q, written by lane i
-    __syncwarp(grp);
-    if (ok)
-        for (int i = 0; i < 4; ++i) Ainv[4 * i + q] = 0.5 * (y[i] + t[i]);
-    __syncwarp(grp);
-    return ok;
+    return 0.5 * (y + __shfl_sync(grp, y, base + 4 * c + r));
 }
 
 // One branch at the current iterate: flows, derivatives, weighted Hessian,
@@ -356,90 +427,113 @@ __device__ __forceinline__ void eval_branch(const DevNet& net, int b, double* W,
     rec[R_S / 2 + 1] = make_double2(St.re, St.im);
 }
 
+// Sum of the block updates u0 .. u1 - 1 for entry (r, c) of their target: sum of L(i,k) U(j,k)^T.
+// The blocks come from the L2 as often as from the L1, so kBatch updates' loads are issued before
+// the first multiply-add.
+__device__ __forceinline__ double run_sum(const DevNet& net, const double* W, const Lay& L, int u0, int u1, int r,
+                                          int c) {
+    double acc = 0.0;
+    const double* Lr = W + L.Lb + 4 * r;
+    const double* Uc = W + L.Ub + 4 * c;
+    int u = u0;
+    for (; u + kBatch <= u1; u += kBatch) {
+        double2 l[kBatch][2], w[kBatch][2];
+#pragma unroll
+        for (int q = 0; q < kBatch; ++q) {
+            const double2* la = reinterpret_cast<const double2*>(Lr + 16 * __ldg(net.sh_a + u + q));
+            const double2* ub = reinterpret_cast<const double2*>(Uc + 16 * __ldg(net.sh_b + u + q));
+            l[q][0] = la[0]; l[q][1] = la[1]; w[q][0] = ub[0]; w[q][1] = ub[1];
+        }
+#pragma unroll
+        for (int q = 0; q < kBatch; ++q)
+            acc += l[q][0].x * w[q][0].x + l[q][0].y * w[q][0].y + l[q][1].x * w[q][1].x + l[q][1].y * w[q][1].y;
+    }
+    for (; u < u1; ++u) {
+        const double2* la = reinterpret_cast<const double2*>(Lr + 16 * __ldg(net.sh_a + u));
+        const double2* ub = reinterpret_cast<const double2*>(Uc + 16 * __ldg(net.sh_b + u));
+        const double2 l0 = la[0], l1 = la[1], w0 = ub[0], w1 = ub[1];
+        acc += l0.x * w0.x + l0.y * w0.y + l1.x * w1.x + l1.y * w1.y;
+    }
+    return acc;
+}
+
 // Solve (L D L^T) v = v in place for the 4-vector-per-bus array v (new order):
 // forward by elimination-tree levels, block diagonal, backward by levels.
+//
+// A narrow level (the top of the tree: 21 of the 118-bus network's 26 levels hold one column)
+// takes a warp per column with eight groups of four lanes: a group takes every eighth block of
+// the column, a lane one of its four rows, and three shuffle additions sum the groups.  An FP64
+// instruction costs its sub-partition 64 cycles with one lane or with 32, so a column of up to
+// eight blocks costs 4 + 3 of them; with a lane per block and the four row sums reduced one after
+// another it was 16 + 20.
 __device__ void ldl_solve(const DevNet& net, const double* W, const Lay& L, double* v) {
     const int tid = threadIdx.x, nb = net.nb, lane = tid & 31, warp = tid >> 5;
+    const int g = lane >> 2, r = lane & 3;
     for (int lev = 0; lev < net.nlevels; ++lev) {
-        const int c0 = net.lev_ptr[lev], c1 = net.lev_ptr[lev + 1];
+        const int c0 = __ldg(net.lev_ptr + lev), c1 = __ldg(net.lev_ptr + lev + 1);
         if (c1 - c0 <= kWarps) {
-            // narrow level (the top of the elimination tree): a warp per column, its
-            // lanes over the blocks of the row, partial sums reduced by shuffles
             if (warp < c1 - c0) {
-                const int j = net.lev_col[c0 + warp];
-                double a0 = 0.0, a1 = 0.0, a2 = 0.0, a3 = 0.0;
-                for (int e = net.Lrowptr[j] + lane; e < net.Lrowptr[j + 1]; e += 32) {
-                    const double* Lq = W + L.Lb + 16 * net.Lrowblk[e];
-                    const double* y = v + 4 * net.Lrowcol[e];
-                    const double y0 = y[0], y1 = y[1], y2 = y[2], y3 = y[3];
-                    a0 += Lq[0] * y0 + Lq[1] * y1 + Lq[2] * y2 + Lq[3] * y3;
-                    a1 += Lq[4] * y0 + Lq[5] * y1 + Lq[6] * y2 + Lq[7] * y3;
-                    a2 += Lq[8] * y0 + Lq[9] * y1 + Lq[10] * y2 + Lq[11] * y3;
-                    a3 += Lq[12] * y0 + Lq[13] * y1 + Lq[14] * y2 + Lq[15] * y3;
+                const int j = __ldg(net.lev_col + c0 + warp);
+                double acc = 0.0;
+                for (int e = __ldg(net.Lrowptr + j) + g; e < __ldg(net.Lrowptr + j + 1); e += 8) {
+                    const double2* Lq = reinterpret_cast<const double2*>(W + L.Lb + 16 * __ldg(net.Lrowblk + e) + 4 * r);
+                    const double2* y = reinterpret_cast<const double2*>(v + 4 * __ldg(net.Lrowcol + e));
+                    const double2 l0 = Lq[0], l1 = Lq[1], y0 = y[0], y1 = y[1];
+                    acc += l0.x * y0.x + l0.y * y0.y + l1.x * y1.x + l1.y * y1.y;
                 }
-                for (int off = 16; off; off >>= 1) {
-                    a0 += __shfl_xor_sync(0xffffffffu, a0, off);
-                    a1 += __shfl_xor_sync(0xffffffffu, a1, off);
-                    a2 += __shfl_xor_sync(0xffffffffu, a2, off);
-                    a3 += __shfl_xor_sync(0xffffffffu, a3, off);
-                }
-                if (lane < 4) v[4 * j + lane] -= (lane == 0 ? a0 : lane == 1 ? a1 : lane == 2 ? a2 : a3);
+                for (int off = 16; off >= 4; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
+                if (lane < 4) v[4 * j + lane] -= acc;
             }
         } else {
             for (int w = tid; w < 4 * (c1 - c0); w += kThreads) {
-                const int j = net.lev_col[c0 + (w >> 2)], r = w & 3;
-                double acc = v[4 * j + r];
-                for (int e = net.Lrowptr[j]; e < net.Lrowptr[j + 1]; ++e) {
-                    const double* Lq = W + L.Lb + 16 * net.Lrowblk[e] + 4 * r;
-                    const double* y = v + 4 * net.Lrowcol[e];
+                const int j = __ldg(net.lev_col + c0 + (w >> 2)), q = w & 3;
+                double acc = v[4 * j + q];
+                for (int e = __ldg(net.Lrowptr + j); e < __ldg(net.Lrowptr + j + 1); ++e) {
+                    const double* Lq = W + L.Lb + 16 * __ldg(net.Lrowblk + e) + 4 * q;
+                    const double* y = v + 4 * __ldg(net.Lrowcol + e);
                     acc -= Lq[0] * y[0] + Lq[1] * y[1] + Lq[2] * y[2] + Lq[3] * y[3];
                 }
-                v[4 * j + r] = acc;
+                v[4 * j + q] = acc;
             }
         }
         __syncthreads();
     }
-    for (int j = tid; j < nb; j += kThreads) {
-        const double* Di = W + L.Di + 16 * j;
-        double* y = v + 4 * j;
-        const double y0 = y[0], y1 = y[1], y2 = y[2], y3 = y[3];
-        for (int r = 0; r < 4; ++r)
-            y[r] = Di[4 * r] * y0 + Di[4 * r + 1] * y1 + Di[4 * r + 2] * y2 + Di[4 * r + 3] * y3;
+    for (int w0 = 0; w0 < 4 * nb; w0 += kThreads) {          // four lanes per bus
+        const int w = w0 + tid, j = w >> 2;
+        double t = 0.0;
+        if (w < 4 * nb) {
+            const double* Di = W + L.Di + 4 * w;             // row w & 3 of block j
+            const double* y = v + 4 * j;
+            t = Di[0] * y[0] + Di[1] * y[1] + Di[2] * y[2] + Di[3] * y[3];
+        }
+        __syncwarp();
+        if (w < 4 * nb) v[w] = t;
     }
     __syncthreads();
     for (int lev = net.nlevels - 1; lev >= 0; --lev) {
-        const int c0 = net.lev_ptr[lev], c1 = net.lev_ptr[lev + 1];
+        const int c0 = __ldg(net.lev_ptr + lev), c1 = __ldg(net.lev_ptr + lev + 1);
         if (c1 - c0 <= kWarps) {
             if (warp < c1 - c0) {
-                const int j = net.lev_col[c0 + warp];
-                double a0 = 0.0, a1 = 0.0, a2 = 0.0, a3 = 0.0;
-                for (int e = net.Lcolptr[j] + lane; e < net.Lcolptr[j + 1]; e += 32) {
-                    const double* Lq = W + L.Lb + 16 * e;
-                    const double* xi = v + 4 * net.Lrow[e];
-                    const double x0 = xi[0], x1 = xi[1], x2 = xi[2], x3 = xi[3];
-                    a0 += Lq[0] * x0 + Lq[4] * x1 + Lq[8] * x2 + Lq[12] * x3;
-                    a1 += Lq[1] * x0 + Lq[5] * x1 + Lq[9] * x2 + Lq[13] * x3;
-                    a2 += Lq[2] * x0 + Lq[6] * x1 + Lq[10] * x2 + Lq[14] * x3;
-                    a3 += Lq[3] * x0 + Lq[7] * x1 + Lq[11] * x2 + Lq[15] * x3;
+                const int j = __ldg(net.lev_col + c0 + warp);
+                double acc = 0.0;
+                for (int e = __ldg(net.Lcolptr + j) + g; e < __ldg(net.Lcolptr + j + 1); e += 8) {
+                    const double* Lq = W + L.Lb + 16 * e + r;
+                    const double* xi = v + 4 * __ldg(net.Lrow + e);
+                    acc += Lq[0] * xi[0] + Lq[4] * xi[1] + Lq[8] * xi[2] + Lq[12] * xi[3];
                 }
-                for (int off = 16; off; off >>= 1) {
-                    a0 += __shfl_xor_sync(0xffffffffu, a0, off);
-                    a1 += __shfl_xor_sync(0xffffffffu, a1, off);
-                    a2 += __shfl_xor_sync(0xffffffffu, a2, off);
-                    a3 += __shfl_xor_sync(0xffffffffu, a3, off);
-                }
-                if (lane < 4) v[4 * j + lane] -= (lane == 0 ? a0 : lane == 1 ? a1 : lane == 2 ? a2 : a3);
+                for (int off = 16; off >= 4; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
+                if (lane < 4) v[4 * j + lane] -= acc;
             }
         } else {
             for (int w = tid; w < 4 * (c1 - c0); w += kThreads) {
-                const int j = net.lev_col[c0 + (w >> 2)], r = w & 3;
-                double acc = v[4 * j + r];
-                for (int e = net.Lcolptr[j]; e < net.Lcolptr[j + 1]; ++e) {
-                    const double* Lq = W + L.Lb + 16 * e + r;
-                    const double* xi = v + 4 * net.Lrow[e];
+                const int j = __ldg(net.lev_col + c0 + (w >> 2)), q = w & 3;
+                double acc = v[4 * j + q];
+                for (int e = __ldg(net.Lcolptr + j); e < __ldg(net.Lcolptr + j + 1); ++e) {
+                    const double* Lq = W + L.Lb + 16 * e + q;
+                    const double* xi = v + 4 * __ldg(net.Lrow + e);
                     acc -= Lq[0] * xi[0] + Lq[4] * xi[1] + Lq[8] * xi[2] + Lq[12] * xi[3];
                 }
-                v[4 * j + r] = acc;
+                v[4 * j + q] = acc;
             }
         }
         __syncthreads();
@@ -448,45 +542,47 @@ __device__ void ldl_solve(const DevNet& net, const double* W, const Lay& L, doub
 
 // r = b - K x with the assembled (unfactored) blocks, one thread per (bus, row),
 // and the componentwise backward error of x, max_i |r_i| / (|K| |x| + |b|)_i
-// (returned per thread, to be max-reduced by the caller).
-__device__ double kkt_residual(const DevNet& net, const double* W, const Lay& L, const double* x, double* r) {
+// (on every thread).  Only the blocks that hold a branch are read: two in three of the
+// factor's blocks are fill, zero in K.
+__device__ double kkt_residual(const DevNet& net, const double* W, const Lay& L, RedBuf& rb, const double* x,
+                               double* r) {
     const int tid = threadIdx.x, nb = net.nb;
-    double worst = 0.0;
+    key_t64 worst = 0;
     for (int w = tid; w < 4 * nb; w += kThreads) {
         const int i = w >> 2, rr = w & 3;
-        const double* Kd = W + L.Kd + 16 * i + 4 * rr;
+        const double* Kd = W + L.Kd + 4 * w;
         const double* xi = x + 4 * i;
-        const double bw = W[L.bv + w];
-        double acc = bw, sc = fabs(bw);
+        double acc = W[L.bv + w], sc = fabs(acc);
+#pragma unroll
         for (int c = 0; c < 4; ++c) {
-            const double t = Kd[c] * xi[c];
-            acc -= t;
-            sc += fabs(t);
+            acc = fma(-Kd[c], xi[c], acc);
+            sc = fma(fabs(Kd[c]), fabs(xi[c]), sc);
         }
-        for (int e = net.Lrowptr[i]; e < net.Lrowptr[i + 1]; ++e) {        // blocks (i, k), k < i
-            const double* Kq = W + L.Kb + 16 * net.Lrowblk[e] + 4 * rr;
-            const double* xk = x + 4 * net.Lrowcol[e];
+        for (int e = __ldg(net.adj_ptr + i); e < __ldg(net.adj_ptr + i + 1); ++e) {
+            const int code = __ldg(net.adj_blk + e);
+            const double* Kq = W + L.Kb + 16 * (code >> 1) + ((code & 1) ? rr : 4 * rr);
+            const int st = (code & 1) ? 4 : 1;
+            const double* xk = x + 4 * __ldg(net.adj_col + e);
+#pragma unroll
             for (int c = 0; c < 4; ++c) {
-                const double t = Kq[c] * xk[c];
-                acc -= t;
-                sc += fabs(t);
-            }
-        }
-        for (int e = net.Lcolptr[i]; e < net.Lcolptr[i + 1]; ++e) {        // blocks (j, i)^T, j > i
-            const double* Kq = W + L.Kb + 16 * e + rr;
-            const double* xj = x + 4 * net.Lrow[e];
-            for (int c = 0; c < 4; ++c) {
-                const double t = Kq[4 * c] * xj[c];
-                acc -= t;
-                sc += fabs(t);
+                const double k = Kq[c * st], xc = xk[c];
+                acc = fma(-k, xc, acc);
+                sc = fma(fabs(k), fabs(xc), sc);
             }
         }
         r[w] = acc;
-        const double be = (sc > 0.0) ? fabs(acc) / sc : (acc == 0.0 ? 0.0 : INFINITY);
-        worst = fmax(worst, isfinite(be) ? be : INFINITY);
+        // |acc| / sc; 0 / 0 counts as 0, a non-finite quotient as infinite
+        key_t64 be = abs_key(sc) > 0 ? abs_key(acc / sc) : (abs_key(acc) ? 0x7ff0000000000000ull : 0ull);
+        if (be > 0x7ff0000000000000ull) be = 0x7ff0000000000000ull;
+        worst = max(worst, be);
     }
+    worst = warp_max_key(worst);
+    if ((tid & 31) == 0) rb.v[0][tid >> 5] = key_value(worst);
     __syncthreads();
-    return worst;
+    worst = 0;
+    for (int w = 0; w < kWarps; ++w) worst = max(worst, abs_key(rb.v[0][w]));
+    __syncthreads();
+    return key_value(worst);
 }
 
 // y = K x with the assembled blocks (x, y: 4-vectors per bus, new order).
@@ -494,18 +590,15 @@ __device__ void kkt_matvec(const DevNet& net, const double* W, const Lay& L, con
     const int tid = threadIdx.x, nb = net.nb;
     for (int w = tid; w < 4 * nb; w += kThreads) {
         const int i = w >> 2, rr = w & 3;
-        const double* Kd = W + L.Kd + 16 * i + 4 * rr;
+        const double* Kd = W + L.Kd + 4 * w;
         const double* xi = x + 4 * i;
         double acc = Kd[0] * xi[0] + Kd[1] * xi[1] + Kd[2] * xi[2] + Kd[3] * xi[3];
-        for (int e = net.Lrowptr[i]; e < net.Lrowptr[i + 1]; ++e) {
-            const double* Kq = W + L.Kb + 16 * net.Lrowblk[e] + 4 * rr;
-            const double* xk = x + 4 * net.Lrowcol[e];
-            acc += Kq[0] * xk[0] + Kq[1] * xk[1] + Kq[2] * xk[2] + Kq[3] * xk[3];
-        }
-        for (int e = net.Lcolptr[i]; e < net.Lcolptr[i + 1]; ++e) {
-            const double* Kq = W + L.Kb + 16 * e + rr;
-            const double* xj = x + 4 * net.Lrow[e];
-            acc += Kq[0] * xj[0] + Kq[4] * xj[1] + Kq[8] * xj[2] + Kq[12] * xj[3];
+        for (int e = __ldg(net.adj_ptr + i); e < __ldg(net.adj_ptr + i + 1); ++e) {
+            const int code = __ldg(net.adj_blk + e);
+            const double* Kq = W + L.Kb + 16 * (code >> 1) + ((code & 1) ? rr : 4 * rr);
+            const int st = (code & 1) ? 4 : 1;
+            const double* xk = x + 4 * __ldg(net.adj_col + e);
+            acc += Kq[0] * xk[0] + Kq[st] * xk[1] + Kq[2 * st] * xk[2] + Kq[3 * st] * xk[3];
         }
         y[w] = acc;
     }
@@ -524,7 +617,7 @@ struct GmresShared {
 // refinement cannot.  Arnoldi with classical Gram-Schmidt applied twice; the
 // candidate solution is formed and its componentwise backward error checked
 // after every step; x ends as the best candidate.  Returns its backward error.
-__device__ double kkt_gmres(const DevNet& net, double* W, const Lay& L, RedBuf& rb, double* red, GmresShared& gs,
+__device__ __noinline__ double kkt_gmres(const DevNet& net, double* W, const Lay& L, RedBuf& rb, double* red, GmresShared& gs,
                             double omega0) {
     const int tid = threadIdx.x, N = 4 * net.nb;
     double* x = W + L.x;
@@ -533,7 +626,7 @@ __device__ double kkt_gmres(const DevNet& net, double* W, const Lay& L, RedBuf& 
     double* V = W + L.kv;
     double* Z = W + L.kz;
     double* t = W + L.gr;
-    const int ops_sum[1] = {1}, ops_max[1] = {0};
+    const int ops_sum[1] = {1};
     int ops_h[kGmresM + 1];
     for (int i = 0; i <= kGmresM; ++i) ops_h[i] = 1;
     {
@@ -620,9 +713,7 @@ __device__ double kkt_gmres(const DevNet& net, double* W, const Lay& L, RedBuf& 
             x[w] = xw;
         }
         __syncthreads();
-        double v1[1] = {kkt_residual(net, W, L, x, t)};
-        block_reduce<1>(rb, v1, ops_max, red);
-        const double om = red[0];
+        const double om = kkt_residual(net, W, L, rb, x, t);
         if (om < best) {
             best = om;
             for (int w = tid; w < N; w += kThreads) xb[w] = x[w];
@@ -738,10 +829,11 @@ __device__ __noinline__ bool dense_solve(const DevNet& net, double* W, const Lay
         unsigned long long m = 0ull;
         auto look = [&](double a, int c) { m = max(m, abs_bits(sc ? a * sc[c] : a)); };
         for (int c = 0; c < 4; ++c) look(W[L.Kd + 16 * i + 4 * (sc ? c : rr) + (sc ? rr : c)], 4 * i + c);
-        for (int e = net.Lrowptr[i]; e < net.Lrowptr[i + 1]; ++e)
-            for (int c = 0; c < 4; ++c) look(W[L.Kb + 16 * net.Lrowblk[e] + 4 * rr + c], 4 * net.Lrowcol[e] + c);
-        for (int e = net.Lcolptr[i]; e < net.Lcolptr[i + 1]; ++e)
-            for (int c = 0; c < 4; ++c) look(W[L.Kb + 16 * e + 4 * c + rr], 4 * net.Lrow[e] + c);
+        for (int e = net.adj_ptr[i]; e < net.adj_ptr[i + 1]; ++e) {
+            const int code = net.adj_blk[e];
+            const double* Kq = W + L.Kb + 16 * (code >> 1) + ((code & 1) ? rr : 4 * rr);
+            for (int c = 0; c < 4; ++c) look(Kq[(code & 1) ? 4 * c : c], 4 * net.adj_col[e] + c);
+        }
         if (m == 0ull) return 1.0;
         int e;
         frexp(__longlong_as_double((long long)m), &e);
@@ -760,6 +852,7 @@ __device__ __noinline__ bool dense_solve(const DevNet& net, double* W, const Lay
     }
     for (int w = tid; w < 16 * net.nL; w += kThreads) {
         const int q = w >> 4, i = 4 * net.Lrow[q] + ((w >> 2) & 3), j = 4 * net.Lcol[q] + (w & 3);
+        if (net.blk_br_ptr[q] == net.blk_br_ptr[q + 1]) continue;      // fill: zero in K
         const double v = W[L.Kb + w];
         A[(long)i * N + j] = v * rs[i] * cs[j];
         A[(long)j * N + i] = v * rs[j] * cs[i];
@@ -991,7 +1084,7 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm)
 opf_kernel(DevNet net, EvalArgs a, const int* islanded, OpfOut o, double tol, int max_it,
            double* scratch, size_t per_cta, Lay L, int* counter) {
     __shared__ RedBuf rb;
-    __shared__ double fsum[kThreads];      // partial update sums of the narrow factorisation levels
+    __shared__ double fsum[2 * kThreads];  // sums of the targets cut between groups (at most 2 per group)
     __shared__ Scal sc;
     const int tid = threadIdx.x;
     double* W = scratch + per_cta * blockIdx.x;
@@ -1326,71 +1419,82 @@ opf_kernel(DevNet net, EvalArgs a, const int* islanded, OpfOut o, double tol, in
                     if (Rb == sc.ref) for (int c = 0; c < 4; ++c) blk[c] = 0.0;
                     if (Cb == sc.ref) for (int r = 0; r < 4; ++r) blk[4 * r] = 0.0;
                     double* U = W + L.Ub + 16 * q;
-                    double* Kq = W + L.Kb + 16 * q;
-                    for (int c = 0; c < 16; ++c) { U[c] = blk[c]; Kq[c] = blk[c]; }
+                    for (int c = 0; c < 16; ++c) U[c] = blk[c];
+                    if (net.blk_br_ptr[q] < net.blk_br_ptr[q + 1]) {     // not fill: kept for the residual
+                        double* Kq = W + L.Kb + 16 * q;
+                        for (int c = 0; c < 16; ++c) Kq[c] = blk[c];
+                    }
                 }
             }
             __syncthreads();
             // ---------------- block LDL^T, level by level ----------------
             for (int lev = 0; lev < net.nlevels; ++lev) {
-                const int t0 = net.tgt_ptr[lev], t1 = net.tgt_ptr[lev + 1], nt = t1 - t0;
-                if (nt > 0 && 32 * nt <= kThreads) {
-                    // few targets (the top of the elimination tree, where each target has the
-                    // longest update lists): S groups of 16 threads per target each sum every
-                    // S-th update, then one thread per entry subtracts the S partial sums
-                    const int S = kThreads / (16 * nt);
-                    if (tid < 16 * nt * S) {
-                        const int ti = tid / (16 * S), g = (tid / 16) % S, e = tid & 15;
-                        const int tg = net.tgt[t0 + ti];
-                        const int r = e >> 2, c = e & 3;
-                        double acc = 0.0;
-                        for (int u = net.upd_ptr[tg] + g; u < net.upd_ptr[tg + 1]; u += S) {
-                            const double* La = W + L.Lb + 16 * net.upd_a[u] + 4 * r;
-                            const double* Ubb = W + L.Ub + 16 * net.upd_b[u] + 4 * c;
-                            acc += La[0] * Ubb[0] + La[1] * Ubb[1] + La[2] * Ubb[2] + La[3] * Ubb[3];
-                        }
-                        fsum[tid] = acc;
+                // A thread per block entry, groups of 16 threads per block.  The level's block updates are
+                // dealt out to the groups in equal shares; a target whose list is cut between groups
+                // collects their sums in shared memory.  On a level with one column (the top of the
+                // tree) the first warp sums and inverts the pivot while the others sum the off-
+                // diagonal blocks.  What bounds it is latency, per level on one scenario: ~5k cycles
+                // for the pivot's updates, ~6k for its inverse, ~3k for the blocks' L; the iteration's
+                // factorisation takes 462k cycles alone (551k with a target per group and four lanes
+                // per pivot), one scenario's OPF 13.1 ms (18.7 with the solves of the same change).
+                const int c0 = net.lev_ptr[lev], nc = net.lev_ptr[lev + 1] - c0;
+                const int e = tid & 15, r = e >> 2, c = e & 3, grp = tid >> 4;
+                const int* rp = net.rn_ptr + lev * kGroups + grp;
+                const bool one = nc == 1 && kGroups > 2;
+                if (one && grp < 2) {
+                    const int j = net.lev_col[c0];
+                    double acc = 0.0;
+                    if (rp[0] < rp[1]) acc = run_sum(net, W, L, net.rn_first[rp[0]], net.rn_first[rp[0] + 1], r, c);
+                    __syncwarp();
+                    acc += __shfl_xor_sync(0xffffffffu, acc, 16);
+                    bool ok;
+                    const double inv = inv4(W[L.Db + 16 * j + e] - acc, 0xffffu << (tid & 16), ok);
+                    if (grp == 0) W[L.Di + 16 * j + e] = inv;
+                    if (!ok) sc.fail = 1;
+                } else {
+                    for (int q = rp[0]; q < rp[1]; ++q) {
+                        const int to = __ldg(net.rn_end + q);
+                        const double acc = run_sum(net, W, L, __ldg(net.rn_first + q), __ldg(net.rn_first + q + 1), r, c);
+                        if (to >= nb) W[L.Ub + 16 * (to - nb) + e] -= acc;
+                        else if (to >= 0) W[L.Db + 16 * to + e] -= acc;
+                        else fsum[16 * (-1 - to) + e] = acc;
+                    }
+                }
+                __syncthreads();
+                if (!one) {
+                    for (int w = tid; w < 4 * nc; w += kThreads) {
+                        const int j = __ldg(net.lev_col + c0 + (w >> 2));
+                        bool ok;
+                        inv4_wide(W + L.Db + 16 * j, W + L.Di + 16 * j, w & 3, 0xfu << (tid & 28), ok);
+                        if (!ok) sc.fail = 1;
                     }
                     __syncthreads();
-                    if (tid < 16 * nt) {
-                        const int ti = tid >> 4, e = tid & 15;
-                        const int tg = net.tgt[t0 + ti];
-                        double* A = (tg < nb) ? (W + L.Db + 16 * tg) : (W + L.Ub + 16 * (tg - nb));
-                        double part = 0.0;
-                        for (int g = 0; g < S; ++g) part += fsum[ti * 16 * S + g * 16 + e];
-                        A[e] -= part;
-                    }
-                } else {
-                    for (int w = tid; w < 16 * nt; w += kThreads) {
-                        const int tg = net.tgt[t0 + (w >> 4)];
-                        const int r = (w & 15) >> 2, c = w & 3;
-                        double* A = (tg < nb) ? (W + L.Db + 16 * tg) : (W + L.Ub + 16 * (tg - nb));
-                        double acc = A[4 * r + c];
-                        for (int u = net.upd_ptr[tg]; u < net.upd_ptr[tg + 1]; ++u) {
-                            const double* La = W + L.Lb + 16 * net.upd_a[u] + 4 * r;
-                            const double* Ubb = W + L.Ub + 16 * net.upd_b[u] + 4 * c;
-                            acc -= La[0] * Ubb[0] + La[1] * Ubb[1] + La[2] * Ubb[2] + La[3] * Ubb[3];
+                }
+                {                                      // L = U D^-1, two blocks of a group at a time
+                    const unsigned m = 0xffffu << (tid & 16);
+                    const int b = (tid & 16) + 4 * r;  // the four lanes of row r
+                    const int o1 = __ldg(net.off_ptr + lev + 1);
+                    for (int o = __ldg(net.off_ptr + lev) + grp; o < o1; o += 2 * kGroups) {
+                        const bool two = o + kGroups < o1;
+                        int4 of[2] = {__ldg(net.off + o), make_int4(0, 0, 0, 0)};
+                        if (two) of[1] = __ldg(net.off + o + kGroups);
+                        double u[2], d[2][4];
+#pragma unroll
+                        for (int q = 0; q < 2; ++q) {
+                            const double* Di = W + L.Di + 16 * of[q].y + c;
+                            u[q] = W[L.Ub + 16 * of[q].x + e];
+                            d[q][0] = Di[0]; d[q][1] = Di[4]; d[q][2] = Di[8]; d[q][3] = Di[12];
                         }
-                        A[4 * r + c] = acc;
+#pragma unroll
+                        for (int q = 0; q < 2; ++q) {
+                            if (q == 1 && !two) break;
+                            for (int p = 0; p < of[q].w; ++p) u[q] -= fsum[16 * (of[q].z + p) + e];
+                            if (of[q].w) W[L.Ub + 16 * of[q].x + e] = u[q];
+                            const double u0 = __shfl_sync(m, u[q], b), u1 = __shfl_sync(m, u[q], b + 1),
+                                         u2 = __shfl_sync(m, u[q], b + 2), u3 = __shfl_sync(m, u[q], b + 3);
+                            W[L.Lb + 16 * of[q].x + e] = u0 * d[q][0] + u1 * d[q][1] + u2 * d[q][2] + u3 * d[q][3];
+                        }
                     }
-                }
-                __syncthreads();
-                {
-                    const int c0 = net.lev_ptr[lev], nc = net.lev_ptr[lev + 1] - c0;
-                    for (int w = tid; w < 4 * nc; w += kThreads) {     // four lanes per pivot
-                        const int j = net.lev_col[c0 + (w >> 2)];
-                        if (!inv4(W + L.Db + 16 * j, W + L.Di + 16 * j, w & 3)) sc.fail = 1;
-                    }
-                }
-                __syncthreads();
-                for (int w = tid; w < 16 * (t1 - t0); w += kThreads) {
-                    const int tg = net.tgt[t0 + (w >> 4)];
-                    if (tg < nb) continue;
-                    const int q = tg - nb;
-                    const int r = (w & 15) >> 2, c = w & 3;
-                    const double* U = W + L.Ub + 16 * q + 4 * r;
-                    const double* Di = W + L.Di + 16 * net.Lcol[q] + c;
-                    W[L.Lb + 16 * q + 4 * r + c] = U[0] * Di[0] + U[1] * Di[4] + U[2] * Di[8] + U[3] * Di[12];
                 }
                 __syncthreads();
             }
@@ -1402,19 +1506,18 @@ opf_kernel(DevNet net, EvalArgs a, const int* islanded, OpfOut o, double tol, in
             // which leaves a low-rank error in the first solve that refinement removes.
             // Refinement stops once the componentwise backward error is at rounding level.
             ldl_solve(net, W, L, W + L.x);
+            double om;
             for (int ref_step = 0;; ++ref_step) {
-                double v1[1] = {kkt_residual(net, W, L, W + L.x, W + L.rv)};
-                const int ops1[1] = {0};
-                block_reduce<1>(rb, v1, ops1, sc.red);
-                if (sc.red[0] <= kRefineTol || ref_step == kRefineSteps) break;   // NaN: refine, then caught below
+                om = kkt_residual(net, W, L, rb, W + L.x, W + L.rv);
+                if (om <= kRefineTol || ref_step == kRefineSteps) break;
                 ldl_solve(net, W, L, W + L.rv);
                 for (int w = tid; w < 4 * nb; w += kThreads) W[L.x + w] += W[L.rv + w];
                 __syncthreads();
             }
-            if (!(sc.red[0] <= kBackwardTol)) {
+            if (!(om <= kBackwardTol)) {
                 // Krylov steps on the factors, then, if those stall, the dense backstop
                 __shared__ GmresShared gs;
-                const double om = kkt_gmres(net, W, L, rb, sc.red, gs, sc.red[0]);
+                om = kkt_gmres(net, W, L, rb, sc.red, gs, om);
                 if (L.dense >= 0 && !(om <= kBackwardTol)) {
                     __shared__ DenseShared ds;
                     if (!dense_solve(net, W, L, ds)) sc.fail = 1;
@@ -1425,10 +1528,7 @@ opf_kernel(DevNet net, EvalArgs a, const int* islanded, OpfOut o, double tol, in
                     // for FP64, and then the backstop's first solution is the best there is)
                     double best = INFINITY;
                     for (int ref_step = 0;; ++ref_step) {
-                        double v1[1] = {kkt_residual(net, W, L, W + L.x, W + L.rv)};
-                        const int ops1[1] = {0};
-                        block_reduce<1>(rb, v1, ops1, sc.red);
-                        const double om_now = sc.red[0];
+                        const double om_now = kkt_residual(net, W, L, rb, W + L.x, W + L.rv);
                         if (ref_step > 0 && !(om_now < best)) {          // no progress: back to the best
                             for (int w = tid; w < 4 * nb; w += kThreads) W[L.x + w] = W[L.gxb + w];
                             __syncthreads();
@@ -1649,6 +1749,8 @@ opf_kernel(DevNet net, EvalArgs a, const int* islanded, OpfOut o, double tol, in
 }
 
 }  // namespace
+
+int opf_groups() { return kGroups; }
 
 int opf_ctas_per_sm() { return kCtasPerSm; }
 

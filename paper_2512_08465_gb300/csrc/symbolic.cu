@@ -184,5 +184,85 @@ std::string symbolic_analysis(int n, const std::vector<int>& f, const std::vecto
         for (int b : bb[q]) S.blk_br.push_back(b);
         S.blk_br_ptr[q + 1] = (int)S.blk_br.size();
     }
+    // per row the blocks that hold a branch (the rest of the pattern is fill, zero in the
+    // assembled matrix): the column, and the block id doubled, odd for the transposed block
+    S.adj_ptr.assign(n + 1, 0);
+    S.adj_col.clear();
+    S.adj_blk.clear();
+    for (int i = 0; i < n; ++i) {
+        for (int e = S.Lrowptr[i]; e < S.Lrowptr[i + 1]; ++e)
+            if (!bb[S.Lrowblk[e]].empty()) {
+                S.adj_col.push_back(S.Lrowcol[e]);
+                S.adj_blk.push_back(2 * S.Lrowblk[e]);
+            }
+        for (int e = S.Lcolptr[i]; e < S.Lcolptr[i + 1]; ++e)
+            if (!bb[e].empty()) {
+                S.adj_col.push_back(S.Lrow[e]);
+                S.adj_blk.push_back(2 * e + 1);
+            }
+        S.adj_ptr[i + 1] = (int)S.adj_col.size();
+    }
     return std::string();
+}
+
+void level_shares(int groups, Symbolic& S) {
+    const int H = S.nlevels;
+    S.rn_ptr.assign((size_t)H * groups + 1, 0);
+    S.rn_first.clear(); S.rn_end.clear();
+    S.sh_a.clear(); S.sh_b.clear();
+    S.off_ptr.assign(H + 1, 0);
+    S.off.clear();
+    std::vector<int> first_slot(S.tgt.size(), 0), slots(S.tgt.size(), 0);
+    for (int h = 0; h < H; ++h) {
+        const int t0 = S.tgt_ptr[h], t1 = S.tgt_ptr[h + 1];
+        const bool one = S.lev_ptr[h + 1] - S.lev_ptr[h] == 1 && groups > 2;
+        int slot = 0;
+        // the updates of the targets `which` (positions in tgt) in shares of groups g0 .. g1 - 1
+        auto deal = [&](const std::vector<int>& which, int g0, int g1, bool diag) {
+            std::vector<int> owner, ua, ub;
+            for (int t : which) {
+                const int tg = S.tgt[t];
+                for (int u = S.upd_ptr[tg]; u < S.upd_ptr[tg + 1]; ++u) {
+                    owner.push_back(t);
+                    ua.push_back(S.upd_a[u]);
+                    ub.push_back(S.upd_b[u]);
+                }
+            }
+            const int U = (int)owner.size();
+            int u0 = 0;
+            for (int q = g0; q < g1; ++q) {
+                S.rn_ptr[(size_t)h * groups + q] = (int)S.rn_end.size();
+                int u1 = std::max(u0, (int)((long long)U * (q - g0 + 1) / (g1 - g0)));
+                while (!one && u1 > 0 && u1 < U && owner[u1] == owner[u1 - 1]) ++u1;
+                for (int u = u0; u < u1; ++u) {
+                    const int t = owner[u];
+                    if (u == u0 || owner[u - 1] != t) S.rn_first.push_back((int)S.sh_a.size());
+                    S.sh_a.push_back(ua[u]);
+                    S.sh_b.push_back(ub[u]);
+                    if (u + 1 < u1 && owner[u + 1] == t) continue;
+                    const bool begun = u0 > 0 && owner[u0 - 1] == t, goes_on = u + 1 < U && owner[u + 1] == t;
+                    if (diag || (!begun && !goes_on)) {
+                        S.rn_end.push_back(S.tgt[t]);
+                    } else {
+                        if (slots[t]++ == 0) first_slot[t] = slot;
+                        S.rn_end.push_back(-1 - slot++);
+                    }
+                }
+                u0 = u1;
+            }
+        };
+        std::vector<int> all, diag;
+        for (int t = t0; t < t1; ++t) (one && S.tgt[t] < S.n ? diag : all).push_back(t);
+        if (one) deal(diag, 0, 2, true);
+        deal(all, one ? 2 : 0, groups, false);
+        for (int t = t0; t < t1; ++t) {
+            const int q = S.tgt[t] - S.n;
+            if (q < 0) continue;
+            const int rec[4] = {q, S.Lcol[q], first_slot[t], slots[t]};
+            S.off.insert(S.off.end(), rec, rec + 4);
+        }
+        S.off_ptr[h + 1] = (int)S.off.size() / 4;
+    }
+    S.rn_ptr[(size_t)H * groups] = (int)S.rn_end.size();
+    S.rn_first.push_back((int)S.sh_a.size());
 }
