@@ -45,14 +45,13 @@ struct Grids {
     int g_opf, g_dyn;
     size_t per_opf, per_dyn;
 };
-constexpr int kDynCtasDefault = 2;
 int cap_opf_of(const cs_ctx* ctx, const Network& net) {
     if (ctx->opt.ctas_per_sm > 0) return ctx->opt.ctas_per_sm;
     return net.opf_cap > 0 ? net.opf_cap : opf_ctas_per_sm();
 }
 int cap_dyn_of(const cs_ctx* ctx, const Network& net) {
     if (ctx->opt.ctas_per_sm > 0) return ctx->opt.ctas_per_sm;
-    return net.dyn_cap > 0 ? net.dyn_cap : kDynCtasDefault;
+    return net.dyn_cap > 0 ? net.dyn_cap : dyn_ctas_per_sm();
 }
 Grids grids(const cs_ctx* ctx, const Network& net, int64_t cn) {
     // persistent kernels sized from occupancy, capped per SM (the network's tuned shape, if any)
@@ -424,11 +423,11 @@ cs_status autotune_network(cs_ctx* ctx, Network* net) {
     const int dyn_try[3] = {1, 2, 4};
     const int tries = std::max(opf_max, 3);
     double best_opf = 1e300, best_dyn = 1e300;
-    int pick_opf = opf_max, pick_dyn = kDynCtasDefault;
+    int pick_opf = opf_max, pick_dyn = dyn_ctas_per_sm();
     const bool was_timing = ctx->timing;
     for (int t = -1; t < tries; ++t) {                 // t = -1: warm-up with the defaults
         net->opf_cap = (t < 0) ? opf_max : 1 + (t % opf_max);
-        net->dyn_cap = (t < 0) ? kDynCtasDefault : dyn_try[t % 3];
+        net->dyn_cap = (t < 0) ? dyn_ctas_per_sm() : dyn_try[t % 3];
         ctx->timing = true;
         ctx->ev_used = 0;
         cs_status st = evaluate_impl(ctx, ctx->direct, net, 0, (const int32_t*)dids.p, (const int32_t*)dids.p + ns,

@@ -186,6 +186,7 @@ cudaError_t launch_dyn(const DevNet& net, const EvalArgs& a, OpfOut o, double da
                        double* scratch, size_t scratch_per_cta, int grid, float* abuf, float* hbuf, double* a64,
                        float* cand, float* hws, int sms, int* counters, int* launches, cudaStream_t s);
 size_t dyn_scratch_doubles(const DevNet& net);
+int dyn_ctas_per_sm();       // resident small-signal CTAs per SM the kernel is built for
 size_t dyn_hbuf_stride(const DevNet& net);
 size_t dyn_abuf_stride(const DevNet& net);
 size_t dyn_a64_stride(const DevNet& net);     // doubles per scenario: the FP64 state matrix (mixed form)

@@ -44,7 +44,8 @@
 
 namespace {
 
-constexpr int kThreads = 256;
+constexpr int kMaxThreads = 512;     // threads of a dyn_kernel block: 128, 256 or 512 (see launch_mode)
+constexpr int kCtasPerSm = 4;        // resident blocks per SM, of 128 threads
 constexpr double kEps = 2.220446049250313e-16;
 // FP32 QR deflates a subdiagonal entry below kDeflTol times its two diagonal neighbours
 // (not the FP32 unit roundoff): the screen's eigenvalues need only be within kEigDelta of
@@ -67,6 +68,7 @@ struct DLay {
     int A;                    // [(5ng)^2]
     int A32;                  // [(5ng)^2] floats (mixed precision screen)
     int wr, wi, v;            // [5ng]
+    int hp;                   // [kHsSlices * 5ng] partial sums of the Hessenberg reduction
     int total;
 };
 constexpr int kGen = 16;      // per-generator doubles: E(2) I(2) e^{jd}(2) Vt(2) |Vt| id iq eq ed ym(2)
@@ -85,6 +87,7 @@ DLay make_dlayout(const DevNet& n) {
     L.A32 = take((25L * n.ng * n.ng + 1) / 2);
     o = (o + 31) & ~31;
     L.wr = take(5L * n.ng); L.wi = take(5L * n.ng); L.v = take(5L * n.ng);
+    L.hp = take(8L * 5 * n.ng);
     L.total = (o + 31) & ~31;
     return L;
 }
@@ -93,35 +96,32 @@ __device__ __forceinline__ cplx ld(const double* p) { return cplx{p[0], p[1]}; }
 __device__ __forceinline__ void st(double* p, cplx v) { p[0] = v.re; p[1] = v.im; }
 
 struct DShared {
-    double red[2][kThreads];
-    int ired[kThreads];
-    double x[3];                     // next bulge column
-    double u[4];                     // reflector of the current step: u0, u1, u2, beta
-    double part[2][kThreads / 32];   // per-warp partial sums, double-buffered
-    int lo, hi, its, fail, scen, m, nn;
-    double hmax;
+    double red[kMaxThreads / 32];
+    int ired[kMaxThreads / 32];
+    double hs[3];                    // Hessenberg reduction: tail, alpha, beta of the current column
+    int fail, scen, m, nn;
     double bal_f;
     int bal_i;
 };
 
 // block reductions ---------------------------------------------------------
 __device__ int bmax_int(DShared& sh, int v) {
-    const int tid = threadIdx.x;
+    const int tid = threadIdx.x, nthr = blockDim.x;
     for (int off = 16; off; off >>= 1) v = max(v, __shfl_xor_sync(0xffffffffu, v, off));
     if ((tid & 31) == 0) sh.ired[tid >> 5] = v;
     __syncthreads();
     int r = sh.ired[0];
-    for (int w = 1; w < kThreads / 32; ++w) r = max(r, sh.ired[w]);
+    for (int w = 1; w < nthr / 32; ++w) r = max(r, sh.ired[w]);
     __syncthreads();
     return r;
 }
 __device__ double bmax(DShared& sh, double v) {
-    const int tid = threadIdx.x;
+    const int tid = threadIdx.x, nthr = blockDim.x;
     for (int off = 16; off; off >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, off));
-    if ((tid & 31) == 0) sh.red[0][tid >> 5] = v;
+    if ((tid & 31) == 0) sh.red[tid >> 5] = v;
     __syncthreads();
-    double r = sh.red[0][0];
-    for (int w = 1; w < kThreads / 32; ++w) r = fmax(r, sh.red[0][w]);
+    double r = sh.red[0];
+    for (int w = 1; w < nthr / 32; ++w) r = fmax(r, sh.red[w]);
     __syncthreads();
     return r;
 }
@@ -166,18 +166,18 @@ __device__ void eig2(double p, double q, double r, double s, double* re, double*
 constexpr int kBalExp = 30;
 template <typename T>
 __device__ void balance(T* A, const int n, T* cs, T* rs, DShared& sh, T* dsc = nullptr) {
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, nthr = blockDim.x, warp = tid >> 5, lane = tid & 31;
     const T fmaxb = (T)ldexp(1.0, sizeof(T) == 8 ? 4 * kBalExp : kBalExp), fminb = (T)1 / fmaxb;
     if (dsc)
-        for (int j = tid; j < n; j += kThreads) dsc[j] = (T)1;
+        for (int j = tid; j < n; j += nthr) dsc[j] = (T)1;
     for (int sweep = 0; sweep < 100; ++sweep) {
-        for (int j = tid; j < n; j += kThreads) {
+        for (int j = tid; j < n; j += nthr) {
             T c = 0;
             for (int i = 0; i < n; ++i)
                 if (i != j) c += fabs(A[(size_t)i * n + j]);
             cs[j] = c;
         }
-        for (int i = warp; i < n; i += kThreads / 32) {
+        for (int i = warp; i < n; i += nthr / 32) {
             T r = 0;
             for (int j = lane; j < n; j += 32)
                 if (j != i) r += fabs(A[(size_t)i * n + j]);
@@ -209,7 +209,7 @@ __device__ void balance(T* A, const int n, T* cs, T* rs, DShared& sh, T* dsc = n
             const int i = sh.bal_i;
             if (i < 0) break;
             const T f = (T)sh.bal_f, finv = (T)(1.0 / sh.bal_f);
-            for (int j = tid; j < n; j += kThreads) {
+            for (int j = tid; j < n; j += nthr) {
                 if (j == i) {
                     cs[i] *= f;
                     rs[i] *= finv;
@@ -230,52 +230,502 @@ __device__ void balance(T* A, const int n, T* cs, T* rs, DShared& sh, T* dsc = n
     }
 }
 
-// Householder reduction to upper Hessenberg form (column k: reflector from
-// rows k+1.., applied from the left to columns k+1.. and from the right to all
-// rows).  The reflector lives in shared memory.
+// Householder reduction to upper Hessenberg form, in place, A row-major n x n in global memory.
+// Column k: reflector v of its rows k+1.., w = beta v^T A, then every row once: left update
+// x = row - v_i w, dot x . v, right update x - beta (x . v) v.  So the matrix is read twice and
+// written once per column (the two updates one after the other read it four times and wrote it
+// twice), the four multiply-adds per entry are the floor, and the row reductions (FP64 additions
+// that fill a warp instruction with one useful lane in the end) go two rows at a time.
+//  * w: the rows in kHsSlices slices, a warp per slice with a lane's columns in registers; the
+//    slices' sums meet in `part` (kHsSlices x n, global).  The slices are fixed, so the sums do not
+//    depend on the number of threads.
+//  * rows: a warp per pair of rows, up to kHsReg * 32 columns in registers; longer rows make the
+//    second pass over memory.
+// The next column is picked up while its rows are written (vn).  v, w, vn: n entries of shared memory.
+constexpr int kHsSlices = 8;
+constexpr int kHsReg = 12;
 template <typename T>
-__device__ void hessenberg(T* A, const int n, T* v, DShared& sh) {
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+__device__ __forceinline__ void sum2(T& a, T& b) {            // both over the warp, to all lanes
+    const bool up = (threadIdx.x & 16) != 0;
+    T mine = up ? b : a, other = up ? a : b;
+    mine += __shfl_xor_sync(0xffffffffu, other, 16);
+    for (int off = 8; off; off >>= 1) mine += __shfl_xor_sync(0xffffffffu, mine, off);
+    other = __shfl_xor_sync(0xffffffffu, mine, 16);
+    a = up ? other : mine;
+    b = up ? mine : other;
+}
+
+template <typename T>
+__device__ __noinline__ void hessenberg(T* A, const int n, T* v, T* w, T* vn, T* part, DShared& sh) {
+    const int tid = threadIdx.x, nthr = blockDim.x, warp = tid >> 5, lane = tid & 31, nw = nthr >> 5;
+    for (int i = tid; i + 1 < n; i += nthr) v[i] = A[(size_t)(i + 1) * n];
+    __syncthreads();
     for (int k = 0; k + 2 < n; ++k) {
-        T t = 0;
-        for (int i = k + 2 + tid; i < n; i += kThreads) {
-            const T q = A[(size_t)i * n + k];
-            t += q * q;
+        const int m = n - k - 1;
+        if (warp == 0) {
+            T t = 0;
+            for (int i = 1 + lane; i < m; i += 32) t += v[i] * v[i];
+            for (int off = 16; off; off >>= 1) t += __shfl_xor_sync(0xffffffffu, t, off);
+            if (lane == 0) {
+                sh.hs[0] = (double)t;
+                if (t != (T)0) {
+                    const T x0 = v[0], nrm = sqrt(x0 * x0 + t), al = (x0 >= (T)0) ? -nrm : nrm, v0 = x0 - al;
+                    v[0] = v0;
+                    sh.hs[1] = (double)al;
+                    sh.hs[2] = (double)((T)2 / (v0 * v0 + t));
+                }
+            }
         }
-        for (int off = 16; off; off >>= 1) t += __shfl_xor_sync(0xffffffffu, t, off);
-        if (lane == 0) sh.part[k & 1][warp] = (double)t;
         __syncthreads();
-        T tail = 0;
-        for (int w = 0; w < kThreads / 32; ++w) tail += (T)sh.part[k & 1][w];
-        if (tail == 0) continue;               // column already reduced (uniform)
-        const T x0 = A[(size_t)(k + 1) * n + k];
-        const T nrm = sqrt(x0 * x0 + tail);
-        const T alpha = (x0 >= 0) ? -nrm : nrm;
-        const T v0 = x0 - alpha;
-        const T beta = (T)2 / (v0 * v0 + tail);
-        const int mm = n - k - 1;
-        for (int i = tid; i < mm; i += kThreads) v[i] = (i == 0) ? v0 : A[(size_t)(k + 1 + i) * n + k];
-        __syncthreads();
-        for (int j = k + 1 + tid; j < n; j += kThreads) {          // left, columns k+1..n-1
-            T* col = A + (size_t)(k + 1) * n + j;
-            T s = 0;
-#pragma unroll 8
-            for (int i = 0; i < mm; ++i) s += v[i] * col[(size_t)i * n];
-            s *= beta;
-#pragma unroll 8
-            for (int i = 0; i < mm; ++i) col[(size_t)i * n] -= s * v[i];
+        T* A1 = A + (size_t)(k + 1) * n + k + 1;               // rows and columns k + 1 ..
+        if (sh.hs[0] == 0.0) {                                 // column already reduced (uniform)
+            for (int i = tid; i + 1 < m; i += nthr) vn[i] = A1[(size_t)(i + 1) * n];
+            __syncthreads();
+            T* q = v; v = vn; vn = q;
+            continue;
         }
-        for (int i = k + 1 + tid; i < n; i += kThreads)            // column k itself
-            A[(size_t)i * n + k] = (i == k + 1) ? alpha : (T)0;
-        __syncthreads();
-        for (int i = warp; i < n; i += kThreads / 32) {            // right, all rows
-            T* row = A + (size_t)i * n + k + 1;
-            T s = 0;
-            for (int j = lane; j < mm; j += 32) s += row[j] * v[j];
-            for (int off = 16; off; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
-            s *= beta;
-            for (int j = lane; j < mm; j += 32) row[j] -= s * v[j];
+        const T alpha = (T)sh.hs[1], beta = (T)sh.hs[2];
+        for (int j0 = 0; j0 < m; j0 += 32 * kHsReg) {
+            for (int sl = warp; sl < kHsSlices; sl += nw) {
+                const int i1 = m * (sl + 1) / kHsSlices;
+                T acc[kHsReg];
+#pragma unroll
+                for (int c = 0; c < kHsReg; ++c) acc[c] = (T)0;
+#pragma unroll 2
+                for (int i = m * sl / kHsSlices; i < i1; ++i) {
+                    const T vi = v[i];
+                    const T* row = A1 + (size_t)i * n + j0 + lane;
+#pragma unroll
+                    for (int c = 0; c < kHsReg; ++c)
+                        if (j0 + 32 * c + lane < m) acc[c] += vi * row[32 * c];
+                }
+#pragma unroll
+                for (int c = 0; c < kHsReg; ++c) {
+                    const int j = j0 + 32 * c + lane;
+                    if (j < m) part[(size_t)sl * n + j] = acc[c];
+                }
+            }
         }
+        __syncthreads();
+        for (int j = tid; j < m; j += nthr) {
+            T t = part[j];
+#pragma unroll
+            for (int sl = 1; sl < kHsSlices; ++sl) t += part[(size_t)sl * n + j];
+            w[j] = beta * t;
+        }
+        __syncthreads();
+        for (int i0 = 2 * warp; i0 < n; i0 += 2 * nw) {
+            T* row[2] = {A + (size_t)i0 * n + k + 1, A + (size_t)min(i0 + 1, n - 1) * n + k + 1};
+            const bool two = i0 + 1 < n;
+            const T vi[2] = {i0 > k ? v[i0 - k - 1] : (T)0, (two && i0 + 1 > k) ? v[i0 - k] : (T)0};
+            T x[2][kHsReg], acc[2] = {(T)0, (T)0};
+            const bool fits = m <= 32 * kHsReg;
+            for (int j0 = 0; j0 < m; j0 += 32 * kHsReg) {
+#pragma unroll
+                for (int c = 0; c < kHsReg; ++c) {
+                    const int j = j0 + 32 * c + lane;
+                    x[0][c] = x[1][c] = (T)0;
+                    if (j < m) {
+                        const T wj = w[j], vj = v[j];
+#pragma unroll
+                        for (int q = 0; q < 2; ++q) {
+                            x[q][c] = row[q][j];
+                            if (i0 + q > k) x[q][c] -= vi[q] * wj;
+                            acc[q] += x[q][c] * vj;
+                        }
+                        if (!fits) {
+                            row[0][j] = x[0][c];
+                            if (two) row[1][j] = x[1][c];
+                        }
+                    }
+                }
+            }
+            sum2(acc[0], acc[1]);
+            acc[0] *= beta;
+            acc[1] *= beta;
+            for (int j0 = 0; j0 < m; j0 += 32 * kHsReg) {
+#pragma unroll
+                for (int c = 0; c < kHsReg; ++c) {
+                    const int j = j0 + 32 * c + lane;
+                    if (j < m) {
+                        const T vj = v[j];
+#pragma unroll
+                        for (int q = 0; q < 2; ++q) {
+                            if (q == 1 && !two) break;
+                            const T y = (fits ? x[q][c] : row[q][j]) - acc[q] * vj;
+                            row[q][j] = y;
+                            if (j == 0 && i0 + q >= k + 2) vn[i0 + q - k - 2] = y;
+                        }
+                    }
+                }
+            }
+            if (lane < (two ? 2 : 1) && i0 + lane > k)
+                A[(size_t)(i0 + lane) * n + k] = (i0 + lane == k + 1) ? alpha : (T)0;
+        }
+        __syncthreads();
+        T* q = v; v = vn; vn = q;
+    }
+}
+
+// One Francis double-shift sweep on rows and columns lo..hi, eigenvalues only, in windows of kQrNB
+// bulge steps:
+//  * chase: one warp carries the bulge through the window with the window's rows in registers, a
+//    lane per column: left reflectors act within a lane, right reflectors act as far as the next
+//    reflector needs them.
+//  * strips: all threads apply the window's kQrNB reflectors to the rest, a thread per row (right
+//    reflectors) and per column to the right (left reflectors), with the row's or column's kQrNB + 2
+//    entries in registers.
+// So a window costs two barriers where a step cost two, and an entry is loaded and stored once per
+// window.  What bounds it is the chase, a chain of dependent instructions of one warp (FP32 ~350
+// cycles a step, FP64 ~2,900; the strips take 100 and 1,000).  118 buses: FP32 QR of one scenario
+// from shared memory 8.2 -> 5.4 ms.
+//
+// Reflector of (x0, x1, x2): I - tau v v^T with v = (1, v1, v2), tau = 1 + |x0| / |x|.
+template <typename T>
+constexpr int kQrNB = sizeof(T) == 8 ? 8 : 12;   // measured: FP32 8 / 12 / 16, FP64 8 / 12 steps
+constexpr int kQrCols = 32;                      // columns of a window kept in the chasing warp
+
+template <typename T>
+struct alignas(16) QrStep {                      // reflector of one step
+    T v1, v2, tau;
+};
+template <typename T>
+struct QrSpace;                                  // in shared memory
+template <>
+struct QrSpace<double> {
+    QrStep<double> st[kQrNB<double>];
+};
+template <>
+struct QrSpace<float> {
+    QrStep<float> st[kQrNB<float>];
+    float blk[kQrNB<float> + 3][kQrNB<float> + 3];             // the window's first columns (odd row stride)
+};
+
+// 1 / sqrt(x) and 1 / x: the hardware approximations in FP32 (2 units in the last place; the
+// reflector's departure from orthogonality stays at rounding level).  In FP64 the FP32 approximation
+// and one step of Halley's iteration (third order: 2^-22 -> 2^-66 relative before rounding), five and
+// three FP64 instructions.  Arguments within 1e-30 .. 1e30.
+__device__ __forceinline__ float qr_rsqrt(float x) {
+    float r;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+__device__ __forceinline__ float qr_rcp(float x) {
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+// (The seeds' conversions run on the integer pipe: an FP64 conversion costs an FP64 instruction.)
+__device__ __forceinline__ float qr_seed(double x) {        // x truncated to FP32
+    const int hi = __double2hiint(x), lo = __double2loint(x);
+    return __int_as_float(((hi - (896 << 20)) << 3) | ((unsigned)lo >> 29));
+}
+__device__ __forceinline__ double qr_wide(float y) {
+    const int b = __float_as_int(y);
+    return __hiloint2double((b >> 3) + (896 << 20), b << 29);
+}
+__device__ __forceinline__ double qr_rsqrt(double x) {
+    const double y = qr_wide(qr_rsqrt(qr_seed(x))), e = fma(-(x * y), y, 1.0);
+    return fma(y * e, fma(0.375, e, 0.5), y);
+}
+__device__ __forceinline__ double qr_rcp(double x) {
+    const double y = qr_wide(qr_rcp(qr_seed(x))), e = fma(-x, y, 1.0);
+    return fma(y, fma(e, e, e), y);
+}
+// x within about 1e-30 .. 1e30 (x a sum of squares: not negative; NaN and infinity are not)
+__device__ __forceinline__ bool qr_safe(float x) { return x > 1e-30f && x < 1e30f; }
+__device__ __forceinline__ bool qr_safe(double x) {
+    return (unsigned)((__double2hiint(x) >> 20) - (1023 - 99)) <= 2u * 99u;
+}
+
+// matrices: row-major in global memory, packed Hessenberg rows in shared memory
+template <typename T>
+struct DenseMat {
+    T* a;
+    int n;
+    __device__ T* at(int i, int j) const { return a + (size_t)i * n + j; }
+};
+template <typename T>
+struct PackedMat {
+    T* a;
+    const int* rb;
+    __device__ T* at(int i, int j) const { return a + rb[i] + j; }
+};
+
+// (x0, x1, x2): the bulge column's entries (x2 = 0 where the row does not exist); its reflector and the
+// column's new first entry.  (x1 = x2 = 0 gives v = 0, tau = 2: a change of sign.)
+template <typename T>
+struct QrRefl {
+    T v1, v2, tau, alpha;
+};
+
+template <typename T>
+__device__ __forceinline__ QrRefl<T> qr_reflector_of(T x0, T x1, T x2, T s) {
+    QrRefl<T> h;
+    const T r = qr_rsqrt(s);
+    h.tau = fabs(x0) * r + (T)1;
+    const T f = copysign(r, x0) * qr_rcp(h.tau);
+    h.v1 = x1 * f;
+    h.v2 = x2 * f;
+    h.alpha = -copysign(s * r, x0);
+    return h;
+}
+
+// out of the range where the squares are safe
+template <typename T>
+__device__ __noinline__ QrRefl<T> qr_reflector_scaled(T x0, T x1, T x2) {
+    const T m = fmax(fabs(x0), fmax(fabs(x1), fabs(x2)));
+    if (!(m > (T)0) || !isfinite(m)) return QrRefl<T>{(T)0, (T)0, (T)0, x0};   // nothing to reflect (or to save)
+    x0 /= m; x1 /= m; x2 /= m;
+    QrRefl<T> h = qr_reflector_of(x0, x1, x2, x0 * x0 + (x1 * x1 + x2 * x2));
+    h.alpha *= m;
+    return h;
+}
+
+template <typename T>
+__device__ __forceinline__ QrRefl<T> qr_reflector(T x0, T x1, T x2) {
+    const T s = x0 * x0 + (x1 * x1 + x2 * x2);
+    if (!qr_safe(s)) return qr_reflector_scaled(x0, x1, x2);
+    return qr_reflector_of(x0, x1, x2, s);
+}
+
+// The bulge between two steps: the entries of its column k - 1 (x, rows k .. k + 2) and the one it
+// fills in column k (b, row k + 2).  They live in registers, never in the matrix.
+template <typename T>
+struct QrBulge {
+    T x0, x1, x2, b;
+};
+
+// Reflectors first .. cnt - 1 on the entries y of one row or column.
+template <bool kFull, typename T>
+__device__ __forceinline__ void qr_apply(T (&y)[kQrNB<T> + 2], const QrSpace<T>& sp, int first, int cnt) {
+#pragma unroll
+    for (int t = 0; t < kQrNB<T>; ++t) {
+        if (!kFull && (t >= cnt || t < first)) continue;
+        const QrStep<T> st = sp.st[t];
+        const T d = st.tau * (y[t] + st.v1 * y[t + 1] + st.v2 * y[t + 2]);
+        y[t] -= d;
+        y[t + 1] -= st.v1 * d;
+        y[t + 2] -= st.v2 * d;
+    }
+}
+
+// Steps kw .. kw + cnt - 1 of the sweep, one warp, the bulge in and out.  Two forms.
+//
+// FP64: the right reflectors are applied to the three rows below the bulge in the lanes too; the
+// nine entries they need are fetched by shuffles, which take less time than an FP64 instruction.
+// The window's rows take the rest of the right reflectors in the strips, each from its own step on.
+template <bool kFull, typename M>
+__device__ __forceinline__ void qr_chase(const M& A, int lo, int hi, int kw, int cnt, QrBulge<double>& bu,
+                                         QrSpace<double>& sp) {
+    const unsigned all = 0xffffffffu;
+    const int lane = threadIdx.x & 31, col = kw + lane;
+    double w[kQrNB<double> + 3];
+#pragma unroll
+    for (int r = 0; r < kQrNB<double> + 3; ++r)
+        w[r] = ((kFull || (kw + r <= hi)) && col <= hi && lane + 1 >= r) ? *A.at(kw + r, col) : 0.0;
+    if (lane == 0) w[2] = bu.b;
+    double x0 = bu.x0, x1 = bu.x1, x2 = bu.x2, sub = 0;   // sub: subdiagonal entry (kw + lane, kw + lane - 1)
+#pragma unroll
+    for (int t = 0; t < kQrNB<double>; ++t) {
+        if (!kFull && t >= cnt) break;
+        const QrRefl<double> h = qr_reflector(x0, x1, x2);
+        const double v1 = h.v1, v2 = h.v2, tau = h.tau, t1 = tau * v1, t2 = tau * v2;
+        if (lane == t) {
+            sub = h.alpha;
+            sp.st[t] = {v1, v2, tau};
+        }
+        const double d = w[t] + v1 * w[t + 1] + v2 * w[t + 2];   // left, rows kw + t ..
+        w[t] -= tau * d;
+        w[t + 1] -= t1 * d;
+        w[t + 2] -= t2 * d;
+        const double a0 = __shfl_sync(all, w[t + 1], t), a1 = __shfl_sync(all, w[t + 1], t + 1),
+                     a2 = __shfl_sync(all, w[t + 1], t + 2);
+        const double b0 = __shfl_sync(all, w[t + 2], t), b1 = __shfl_sync(all, w[t + 2], t + 1),
+                     b2 = __shfl_sync(all, w[t + 2], t + 2);
+        const double da = a0 + v1 * a1 + v2 * a2, db = b0 + v1 * b1 + v2 * b2, dc = v2 * __shfl_sync(all, w[t + 3], t + 2);
+        const double co = lane == t ? tau : lane == t + 1 ? t1 : lane == t + 2 ? t2 : 0.0;
+        w[t + 1] -= co * da;
+        w[t + 2] -= co * db;
+        w[t + 3] -= co * dc;
+        x0 = __shfl_sync(all, w[t + 1], t);
+        x1 = __shfl_sync(all, w[t + 2], t);
+        x2 = __shfl_sync(all, w[t + 3], t);
+    }
+    bu = QrBulge<double>{x0, x1, x2, kFull ? __shfl_sync(all, w[kQrNB<double> + 2], kQrNB<double>) : 0.0};
+    // a column of the window is final on and above its diagonal; its subdiagonal entry is the next
+    // step's alpha (the last one's, the next window's, or x0 at the end of the sweep)
+#pragma unroll
+    for (int r = 0; r < kQrNB<double> + 3; ++r)
+        if ((kFull || kw + r <= hi) && col <= hi && (lane >= r || (lane + 1 == r && lane >= cnt)))
+            *A.at(kw + r, col) = w[r];
+    if (lane < cnt && col > lo) *A.at(col, col - 1) = sub;
+    if (kw + cnt == hi && lane == 0) *A.at(hi, hi - 1) = x0;
+}
+
+// FP32: the lanes take the left reflectors only (left and right ones commute), and the chain from one
+// reflector to the next runs on copies of its few entries that every lane keeps: rows k .. k + 2 of
+// columns k and k + 1, and column k + 2, fetched before the reflector is known.  So no shuffle lies on
+// the chain and a step is ~50 instructions of one warp.  The right reflectors act on the window's
+// first columns in the strips (sp.blk holds them meanwhile, with the entries that the left reflectors
+// fill below the subdiagonal).
+template <bool kFull, typename M>
+__device__ __forceinline__ void qr_chase(const M& A, int lo, int hi, int kw, int cnt, QrBulge<float>& bu,
+                                         QrSpace<float>& sp) {
+    const unsigned all = 0xffffffffu;
+    const int lane = threadIdx.x & 31, col = kw + lane;
+    float w[kQrNB<float> + 3];
+#pragma unroll
+    for (int r = 0; r < kQrNB<float> + 3; ++r)
+        w[r] = ((kFull || (kw + r <= hi)) && col <= hi && lane + 1 >= r) ? *A.at(kw + r, col) : 0.0f;
+    if (lane == 0) w[2] = bu.b;
+    float x0 = bu.x0, x1 = bu.x1, x2 = bu.x2, sub = 0;    // sub: subdiagonal entry (kw + lane, kw + lane - 1)
+    float m00 = __shfl_sync(all, w[0], 0), m01 = __shfl_sync(all, w[0], 1);
+    float m10 = __shfl_sync(all, w[1], 0), m11 = __shfl_sync(all, w[1], 1);
+    float m20 = bu.b, m21 = __shfl_sync(all, w[2], 1);
+#pragma unroll
+    for (int t = 0; t < kQrNB<float>; ++t) {
+        if (!kFull && t >= cnt) break;
+        const float c0 = __shfl_sync(all, w[t], t + 2), c1 = __shfl_sync(all, w[t + 1], t + 2),
+                    c2 = __shfl_sync(all, w[t + 2], t + 2), s3 = __shfl_sync(all, w[t + 3], t + 2);
+        const QrRefl<float> h = qr_reflector(x0, x1, x2);
+        const float v1 = h.v1, v2 = h.v2, tau = h.tau, t1 = tau * v1, t2 = tau * v2;
+        sp.st[t] = {v1, v2, tau};                         // the same from every lane
+        if (lane == t) sub = h.alpha;
+        const float d0 = m00 + v1 * m10 + v2 * m20, d1 = m01 + v1 * m11 + v2 * m21, d2 = c0 + v1 * c1 + v2 * c2;
+        const float n10 = m10 - t1 * d0, n20 = m20 - t2 * d0, n11 = m11 - t1 * d1, n21 = m21 - t2 * d1,
+                    n12 = c1 - t1 * d2, n22 = c2 - t2 * d2;
+        const float da = n10 + v1 * n11 + v2 * n12, db = n20 + v1 * n21 + v2 * n22, dc = v2 * s3;
+        x0 = n10 - tau * da;
+        x1 = n20 - tau * db;
+        x2 = -(tau * dc);
+        m00 = n11 - t1 * da; m01 = n12 - t2 * da;
+        m10 = n21 - t1 * db; m11 = n22 - t2 * db;
+        m20 = -(t1 * dc);    m21 = s3 - t2 * dc;
+        const float d = w[t] + v1 * w[t + 1] + v2 * w[t + 2];     // left, rows kw + t ..
+        w[t] -= tau * d;
+        w[t + 1] -= t1 * d;
+        w[t + 2] -= t2 * d;
+    }
+    bu = QrBulge<float>{x0, x1, x2, m20};
+    if (lane < kQrNB<float> + 2) {
+#pragma unroll
+        for (int r = 0; r < kQrNB<float> + 3; ++r) sp.blk[r][lane] = w[r];
+    } else if (col <= hi) {                               // right of the reflectors' columns: final
+#pragma unroll
+        for (int r = 0; r < kQrNB<float> + 3; ++r)
+            if ((kFull || kw + r <= hi) && lane + 1 >= r) *A.at(kw + r, col) = w[r];
+    }
+    if (lane < cnt && col > lo) *A.at(col, col - 1) = sub;
+    if (kw + cnt == hi && lane == 0) *A.at(hi, hi - 1) = x0;
+}
+
+// The window's own rows in the strips: FP64, from the matrix, each row from its own step on; FP32, from
+// sp.blk, all of them.
+template <typename M>
+__device__ __forceinline__ void qr_own_rows(const M& A, int hi, int kw, int cnt, const QrSpace<double>& sp, int lane) {
+    if (lane >= cnt) return;
+    double y[kQrNB<double> + 2];
+    double* row = A.at(kw + lane, kw);
+#pragma unroll
+    for (int c = 0; c < kQrNB<double> + 2; ++c) y[c] = (c >= lane && c <= cnt + 1 && kw + c <= hi) ? row[c] : 0.0;
+    qr_apply<false>(y, sp, lane, cnt);
+#pragma unroll
+    for (int c = 0; c < kQrNB<double> + 2; ++c)
+        if (c >= lane && c <= cnt + 1 && kw + c <= hi) row[c] = y[c];
+}
+template <typename M>
+__device__ __forceinline__ void qr_own_rows(const M& A, int hi, int kw, int cnt, const QrSpace<float>& sp, int lane) {
+    if (lane >= kQrNB<float> + 3 || kw + lane > hi) return;
+    float y[kQrNB<float> + 2];
+#pragma unroll
+    for (int c = 0; c < kQrNB<float> + 2; ++c) y[c] = sp.blk[lane][c];
+    if (cnt == kQrNB<float>) qr_apply<true>(y, sp, 0, kQrNB<float>);
+    else qr_apply<false>(y, sp, 0, cnt);
+    float* row = A.at(kw + lane, kw);
+    // on and right of the diagonal; below it only the entries right of the bulge column (the
+    // others are the steps' alphas and zeros)
+#pragma unroll
+    for (int c = 0; c < kQrNB<float> + 2; ++c)
+        if (kw + c <= hi && (c >= lane || (c + 1 == lane && c >= cnt))) row[c] = y[c];
+}
+
+// The window's reflectors on the rows above it, the columns right of it, and its own rows (each from
+// its own step on).  A warp takes 32 rows or 32 columns at a time.
+template <typename T, typename M>
+__device__ __forceinline__ void qr_strips(const M& A, int lo, int hi, int kw, int cnt, const QrSpace<T>& sp, int warp,
+                                          int nwarps) {
+    const int lane = threadIdx.x & 31, nrow = kw - lo, jc = kw + kQrCols, ncol = max(0, hi + 1 - jc);
+    const int trow = (nrow + 31) >> 5, tcol = (ncol + 31) >> 5;
+    const bool full = cnt == kQrNB<T> && kw + kQrNB<T> + 1 <= hi;
+    for (int task = warp; task < trow + tcol + 1; task += nwarps) {
+        T y[kQrNB<T> + 2];
+        if (task < trow) {
+            const int i = lo + 32 * task + lane;
+            if (i >= kw) continue;
+            T* row = A.at(i, kw);
+            if (full) {
+#pragma unroll
+                for (int c = 0; c < kQrNB<T> + 2; ++c) y[c] = row[c];
+                qr_apply<true>(y, sp, 0, kQrNB<T>);
+#pragma unroll
+                for (int c = 0; c < kQrNB<T> + 2; ++c) row[c] = y[c];
+            } else {
+#pragma unroll
+                for (int c = 0; c < kQrNB<T> + 2; ++c) y[c] = (c <= cnt + 1 && kw + c <= hi) ? row[c] : (T)0;
+                qr_apply<false>(y, sp, 0, cnt);
+#pragma unroll
+                for (int c = 0; c < kQrNB<T> + 2; ++c)
+                    if (c <= cnt + 1 && kw + c <= hi) row[c] = y[c];
+            }
+        } else if (task < trow + tcol) {                         // (columns right of a window: it is full)
+            const int j = jc + 32 * (task - trow) + lane;
+            if (j > hi) continue;
+#pragma unroll
+            for (int r = 0; r < kQrNB<T> + 2; ++r) y[r] = *A.at(kw + r, j);
+            qr_apply<true>(y, sp, 0, kQrNB<T>);
+#pragma unroll
+            for (int r = 0; r < kQrNB<T> + 2; ++r) *A.at(kw + r, j) = y[r];
+        } else {
+            qr_own_rows(A, hi, kw, cnt, sp, lane);
+        }
+    }
+}
+
+// First column of the double-shift step: (H^2 - s H + t I) e1 of the block lo..hi, with the shifts'
+// sum s and product t from its trailing 2x2 block or, if exceptional, from its last subdiagonals.
+template <typename T, typename M>
+__device__ __forceinline__ void qr_start(const M& A, int lo, int hi, bool exceptional, QrBulge<T>& bu) {
+    const T a11 = *A.at(hi - 1, hi - 1), a12 = *A.at(hi - 1, hi), a21 = *A.at(hi, hi - 1), a22 = *A.at(hi, hi);
+    T sft = a11 + a22, tft = a11 * a22 - a12 * a21;
+    if (exceptional) {
+        const T ww = fabs(a21) + fabs(*A.at(hi - 1, hi - 2));
+        sft = (T)1.5 * ww;
+        tft = ww * ww;
+    }
+    const T h00 = *A.at(lo, lo), h01 = *A.at(lo, lo + 1), h10 = *A.at(lo + 1, lo), h11 = *A.at(lo + 1, lo + 1);
+    bu.x0 = h00 * h00 + h01 * h10 - sft * h00 + tft;
+    bu.x1 = h10 * (h00 + h11 - sft);
+    bu.x2 = h10 * *A.at(lo + 2, lo + 1);
+    bu.b = (T)0;
+}
+
+// Whole sweep by the block: the warp `chaser` starts and chases, all threads take the strips.
+template <typename T, typename M>
+__device__ __forceinline__ void qr_sweep(const M& A, int lo, int hi, bool exceptional, QrSpace<T>& sp, int nthreads,
+                                         int chaser) {
+    const int tid = threadIdx.x, nthr = blockDim.x;
+    const bool mine = (tid >> 5) == chaser;
+    QrBulge<T> bu{};
+    if (mine) qr_start<T>(A, lo, hi, exceptional, bu);
+    for (int kw = lo; kw < hi; kw += kQrNB<T>) {
+        const int cnt = min(kQrNB<T>, hi - kw);
+        if (mine) {
+            if (kw + kQrNB<T> + 2 <= hi) qr_chase<true>(A, lo, hi, kw, cnt, bu, sp);
+            else qr_chase<false>(A, lo, hi, kw, cnt, bu, sp);
+        }
+        __syncthreads();
+        qr_strips<T>(A, lo, hi, kw, cnt, sp, tid >> 5, nthreads >> 5);
         __syncthreads();
     }
 }
@@ -284,151 +734,66 @@ __device__ void hessenberg(T* A, const int n, T* v, DShared& sh) {
 // eigenvalues only (updates restricted to the active block lo..hi).
 // sh.fail = 2 if it does not converge in 30 n sweeps.
 template <typename T>
-__device__ void hqr_global(T* A, const int n, double* wr, double* wi, DShared& sh) {
-    const int tid = threadIdx.x;
-    const double eps = (sizeof(T) == 8) ? kEps : (double)kDeflTol;       // deflation tolerance
+__device__ __noinline__ void hqr_global(T* Ag, const int n, double* wr, double* wi, DShared& sh) {
+    __shared__ QrSpace<T> sp;
+    const int tid = threadIdx.x, nthr = blockDim.x;
+    const DenseMat<T> A{Ag, n};
+    // The blocks resident on an SM chase with different warps: an FP64 chase fills its sub-partition's
+    // FP64 pipe, and warp w of a block sits on sub-partition w mod 4 (consecutive blocks, or blocks one
+    // grid round apart, share an SM).
+    const int chaser = (blockIdx.x + blockIdx.x / 152) & 3;
+    const T eps = (sizeof(T) == 8) ? (T)kEps : (T)kDeflTol;              // deflation tolerance
+    double hmax;
     {
         double hm = 0.0;
-        for (int w = tid; w < n * n; w += kThreads) {
-            const int i = w / n, j = w % n;
-            if (j >= i - 1) hm = fmax(hm, fabs((double)A[w]));
-        }
-        hm = bmax(sh, hm);
-        if (tid == 0) {
-            sh.hmax = hm;
-            sh.hi = n - 1;
-            sh.its = 0;
-        }
-        __syncthreads();
+        for (int i = tid >> 5; i < n; i += nthr / 32)
+            for (int j = max(0, i - 1) + (tid & 31); j < n; j += 32) hm = fmax(hm, fabs((double)*A.at(i, j)));
+        hmax = bmax(sh, hm);
     }
-    while (sh.hi >= 0) {
-        const int hi = sh.hi;
+    int hi = n - 1, its = 0;
+    while (hi >= 0) {
         // top of the unreduced block ending at hi: largest l <= hi with a negligible A[l][l-1]
         int cand = 0;
-        for (int l = 1 + tid; l <= hi; l += kThreads) {
-            double sd = fabs((double)A[(size_t)(l - 1) * n + l - 1]) + fabs((double)A[(size_t)l * n + l]);
-            if (sd == 0.0) sd = sh.hmax;
-            if (fabs((double)A[(size_t)l * n + l - 1]) <= eps * sd) cand = max(cand, l);
+        for (int l = 1 + tid; l <= hi; l += nthr) {
+            T sd = fabs(*A.at(l - 1, l - 1)) + fabs(*A.at(l, l));
+            if (sd == (T)0) sd = (T)hmax;
+            if (fabs(*A.at(l, l - 1)) <= eps * sd) cand = max(cand, l);
         }
         const int lo = bmax_int(sh, cand);
         if (lo == hi) {
             if (tid == 0) {
-                wr[hi] = A[(size_t)hi * n + hi];
+                wr[hi] = *A.at(hi, hi);
                 wi[hi] = 0.0;
-                sh.hi = hi - 1;
-                sh.its = 0;
             }
-            __syncthreads();
+            hi -= 1;
+            its = 0;
             continue;
         }
         if (lo == hi - 1) {
             if (tid == 0) {
                 double re[2], im[2];
-                eig2(A[(size_t)(hi - 1) * n + hi - 1], A[(size_t)(hi - 1) * n + hi], A[(size_t)hi * n + hi - 1],
-                     A[(size_t)hi * n + hi], re, im);
+                eig2(*A.at(hi - 1, hi - 1), *A.at(hi - 1, hi), *A.at(hi, hi - 1), *A.at(hi, hi), re, im);
                 wr[hi - 1] = re[0]; wi[hi - 1] = im[0];
                 wr[hi] = re[1]; wi[hi] = im[1];
-                sh.hi = hi - 2;
-                sh.its = 0;
             }
-            __syncthreads();
+            hi -= 2;
+            its = 0;
             continue;
         }
-        if (sh.its >= 30 * n) {
+        if (its >= 30 * n) {
             if (tid == 0) sh.fail = 2;
-            __syncthreads();
             break;
         }
-        __syncthreads();
-        if (tid == 0) {
-            const int its = ++sh.its;
-            double sft, tft;
-            const double a11 = A[(size_t)(hi - 1) * n + hi - 1], a12 = A[(size_t)(hi - 1) * n + hi];
-            const double a21 = A[(size_t)hi * n + hi - 1], a22 = A[(size_t)hi * n + hi];
-            if (its == 10 || its == 20) {              // exceptional shift
-                const double ww = fabs(a21) + fabs(A[(size_t)(hi - 1) * n + hi - 2]);
-                sft = 1.5 * ww;
-                tft = ww * ww;
-            } else {
-                sft = a11 + a22;
-                tft = a11 * a22 - a12 * a21;
-            }
-            const double h00 = A[(size_t)lo * n + lo], h01 = A[(size_t)lo * n + lo + 1];
-            const double h10 = A[(size_t)(lo + 1) * n + lo], h11 = A[(size_t)(lo + 1) * n + lo + 1];
-            const double h21 = A[(size_t)(lo + 2) * n + lo + 1];
-            sh.x[0] = h00 * h00 + h01 * h10 - sft * h00 + tft;
-            sh.x[1] = h10 * (h00 + h11 - sft);
-            sh.x[2] = h10 * h21;
-        }
-        __syncthreads();
-        // The reflector of each step is computed once, by thread 0, and broadcast: on this
-        // GPU a warp-wide FP64 instruction costs the FP64 pipe the same whatever its active
-        // lanes, so every warp computing it would multiply that cost by the warp count.
-        for (int k = lo; k <= hi - 1; ++k) {
-            const int len = (k + 2 <= hi) ? 3 : 2;
-            const bool more = (k + 1 <= hi - 1);
-            if (tid == 0) {
-                const double x0 = sh.x[0], x1 = sh.x[1], x2 = (len == 3) ? sh.x[2] : 0.0;
-                const double t2 = x1 * x1 + x2 * x2;
-                if (t2 != 0.0) {
-                    const double nrm = sqrt(x0 * x0 + t2);
-                    const double al = (x0 >= 0.0) ? -nrm : nrm;
-                    sh.u[0] = x0 - al;
-                    sh.u[1] = x1;
-                    sh.u[2] = x2;
-                    sh.u[3] = 2.0 / ((x0 - al) * (x0 - al) + t2);
-                } else {
-                    sh.u[3] = 0.0;                 // no reflector this step
-                }
-            }
-            __syncthreads();
-            const T bt = (T)sh.u[3];
-            if (bt != (T)0) {
-                const T u0 = (T)sh.u[0], u1 = (T)sh.u[1], u2 = (len == 3) ? (T)sh.u[2] : (T)0;
-                const int c0 = (k > lo) ? k - 1 : lo;
-                for (int j = c0 + tid; j <= hi; j += kThreads) {   // rows k..k+len-1
-                    T* p0 = A + (size_t)k * n + j;
-                    T d = u0 * p0[0] + u1 * p0[n];
-                    if (len == 3) d += u2 * p0[2 * n];
-                    d *= bt;
-                    p0[0] -= d * u0;
-                    p0[n] -= d * u1;
-                    if (len == 3) p0[2 * n] -= d * u2;
-                }
-                __syncthreads();
-                const int r1 = (k + 3 < hi) ? k + 3 : hi;
-                for (int i = lo + tid; i <= r1; i += kThreads) {   // columns k..k+len-1
-                    T* p0 = A + (size_t)i * n + k;
-                    T d = p0[0] * u0 + p0[1] * u1;
-                    if (len == 3) d += p0[2] * u2;
-                    d *= bt;
-                    p0[0] -= d * u0;
-                    p0[1] -= d * u1;
-                    if (len == 3) p0[2] -= d * u2;
-                    if (i > k && i <= k + 3) sh.x[i - k - 1] = (double)p0[0];   // next bulge column
-                }
-                __syncthreads();
-            } else if (more) {
-                if (tid == 0) {
-                    sh.x[0] = A[(size_t)(k + 1) * n + k];
-                    sh.x[1] = A[(size_t)(k + 2) * n + k];
-                    sh.x[2] = (k + 3 <= hi) ? (double)A[(size_t)(k + 3) * n + k] : 0.0;
-                }
-                __syncthreads();
-            }
-        }
-        for (int i = lo + 2 + tid; i <= hi; i += kThreads) {
-            A[(size_t)i * n + i - 2] = (T)0;
-            if (i >= lo + 3) A[(size_t)i * n + i - 3] = (T)0;
-        }
-        __syncthreads();
+        ++its;
+        qr_sweep<T>(A, lo, hi, its == 10 || its == 20, sp, nthr, chaser);
     }
+    __syncthreads();                               // eigenvalues and sh.fail written by thread 0
 }
 
 template <typename T>
-__device__ void eigen_screen(T* A, const int n, T* cs, T* rs, T* v, double* wr, double* wi, DShared& sh) {
+__device__ void eigen_screen(T* A, const int n, T* cs, T* rs, T* v, T* part, double* wr, double* wi, DShared& sh) {
     balance<T>(A, n, cs, rs, sh);
-    hessenberg<T>(A, n, v, sh);
+    hessenberg<T>(A, n, v, cs, rs, part, sh);
     hqr_global<T>(A, n, wr, wi, sh);
 }
 
@@ -473,10 +838,10 @@ constexpr double kRefinedGuard = 1e-7;
 
 // max Re and min damping ratio over the n eigenvalues (block-wide, result on all threads)
 __device__ void eig_stats(DShared& sh, int n, const double* wr, const double* wi, double& maxre, double& minz) {
-    const int tid = threadIdx.x;
+    const int tid = threadIdx.x, nthr = blockDim.x;
     double mr = -INFINITY, mz = INFINITY;
     if (!sh.fail) {
-        for (int i = tid; i < n; i += kThreads) {
+        for (int i = tid; i < n; i += nthr) {
             mr = fmax(mr, wr[i]);
             const double mg = sqrt(wr[i] * wr[i] + wi[i] * wi[i]);
             mz = fmin(mz, mg > 0.0 ? -wr[i] / mg : 1.0);
@@ -501,7 +866,7 @@ __device__ void eig_stats(DShared& sh, int n, const double* wr, const double* wi
 enum { DYN_FULL64 = 0, DYN_MIXED_INLINE = 1, DYN_FRONT = 2, DYN_RERUN = 3, DYN_FRONT_LARGE = 4, DYN_QR_LARGE = 5 };
 
 template <int kMode>
-__global__ void __launch_bounds__(kThreads)
+__global__ void __launch_bounds__(kMaxThreads, 1)
 dyn_kernel(DevNet net, EvalArgs a, OpfOut o, double damping_min, double* scratch, size_t per_cta, DLay L,
            float* hbuf, size_t hstride, double* a64, size_t a64stride, int* counter) {
     __shared__ DShared sh;
@@ -510,7 +875,7 @@ dyn_kernel(DevNet net, EvalArgs a, OpfOut o, double damping_min, double* scratch
     double* cs_d = dsm + ((net.ng + 1) >> 1);
     double* rs_d = cs_d + 5 * net.ng;
     double* v_d = rs_d + 5 * net.ng;
-    const int tid = threadIdx.x;
+    const int tid = threadIdx.x, nthr = blockDim.x;
     double* W = scratch + per_cta * blockIdx.x;
     const int nb = net.nb, ng = net.ng, nbr = net.nbr;
     const int nx = 2 * nb + 2 * ng;
@@ -577,7 +942,7 @@ dyn_kernel(DevNet net, EvalArgs a, OpfOut o, double damping_min, double* scratch
         const int m = sh.m, n = sh.nn;
 
         // ---- 1. assemble Y_bb on the symbolic pattern ----
-        for (int tg = tid; tg < nb + net.nL; tg += kThreads) {
+        for (int tg = tid; tg < nb + net.nL; tg += nthr) {
             if (tg < nb) {
                 const int j = tg, i = net.perm[j];
                 if (!live(i)) {                       // de-energised bus: identity row
@@ -615,7 +980,7 @@ dyn_kernel(DevNet net, EvalArgs a, OpfOut o, double damping_min, double* scratch
         // ---- complex LDL^T, level by level ----
         for (int lev = 0; lev < net.nlevels; ++lev) {
             const int t0 = net.tgt_ptr[lev], t1 = net.tgt_ptr[lev + 1];
-            for (int w = tid; w < t1 - t0; w += kThreads) {
+            for (int w = tid; w < t1 - t0; w += nthr) {
                 const int tg = net.tgt[t0 + w];
                 double* A = (tg < nb) ? (W + L.Yd + 2 * tg) : (W + L.Yu + 2 * (tg - nb));
                 cplx acc = ld(A);
@@ -624,14 +989,14 @@ dyn_kernel(DevNet net, EvalArgs a, OpfOut o, double damping_min, double* scratch
                 st(A, acc);
             }
             __syncthreads();
-            for (int w = net.lev_ptr[lev] + tid; w < net.lev_ptr[lev + 1]; w += kThreads) {
+            for (int w = net.lev_ptr[lev] + tid; w < net.lev_ptr[lev + 1]; w += nthr) {
                 const int j = net.lev_col[w];
                 const cplx d = ld(W + L.Yd + 2 * j);
                 if (!(abs2(d) > 0.0) || !isfinite(abs2(d))) sh.fail = 1;
                 st(W + L.Ydi + 2 * j, cdiv(cm(1.0, 0.0), d));
             }
             __syncthreads();
-            for (int w = tid; w < t1 - t0; w += kThreads) {
+            for (int w = tid; w < t1 - t0; w += nthr) {
                 const int tg = net.tgt[t0 + w];
                 if (tg < nb) continue;
                 const int q = tg - nb;
@@ -640,7 +1005,7 @@ dyn_kernel(DevNet net, EvalArgs a, OpfOut o, double damping_min, double* scratch
             __syncthreads();
         }
         // ---- 2. machine-bus entries of Y_bb^{-1}: one sparse solve per machine ----
-        for (int kk = tid; kk < m; kk += kThreads) {
+        for (int kk = tid; kk < m; kk += nthr) {
             double* y = W + L.rhs + (size_t)2 * nb * kk;
             for (int j = 0; j < nb; ++j) { y[2 * j] = 0.0; y[2 * j + 1] = 0.0; }
             const int jb = net.iperm[net.gbus[gidx[kk]]];
@@ -661,7 +1026,7 @@ dyn_kernel(DevNet net, EvalArgs a, OpfOut o, double damping_min, double* scratch
         }
         __syncthreads();
         // Y_red[k][l] = ym_k delta_kl - ym_k ym_l (Ybb^-1)[b_k][b_l]
-        for (int w = tid; w < m * m; w += kThreads) {
+        for (int w = tid; w < m * m; w += nthr) {
             const int k = w / m, l = w % m;
             const cplx ymk = cm(0.0, -1.0 / net.xp[gidx[k]]), yml = cm(0.0, -1.0 / net.xp[gidx[l]]);
             const int jl = net.iperm[net.gbus[gidx[l]]];
@@ -671,7 +1036,7 @@ dyn_kernel(DevNet net, EvalArgs a, OpfOut o, double damping_min, double* scratch
             st(W + L.Z + 2 * (size_t)(k * m + l), v);
         }
         // ---- 3. equilibrium per machine ----
-        for (int kk = tid; kk < m; kk += kThreads) {
+        for (int kk = tid; kk < m; kk += nthr) {
             const int k = gidx[kk], i = net.gbus[k];
             double sa, ca;
             sincos(xs[i], &sa, &ca);
@@ -698,7 +1063,7 @@ dyn_kernel(DevNet net, EvalArgs a, OpfOut o, double damping_min, double* scratch
         __syncthreads();
         // network currents at the equilibrium state: I = Y_red E' (the OPF injection up
         // to the OPF residual), and the dq currents and terminal voltage from them
-        for (int kk = tid; kk < m; kk += kThreads) {
+        for (int kk = tid; kk < m; kk += nthr) {
             double* g = W + L.gen + kGen * kk;
             cplx I = cm(0.0, 0.0);
             for (int ll = 0; ll < m; ++ll)
@@ -716,7 +1081,7 @@ dyn_kernel(DevNet net, EvalArgs a, OpfOut o, double damping_min, double* scratch
         // ---- state matrix: one thread per 5x5 block (k, l) ----
         // (the front kernel keeps it per scenario for the FP64 refinement)
         double* A = (kMode == DYN_FRONT && a64) ? a64 + (size_t)s * a64stride : W + L.A;
-        for (int w = tid; w < m * m; w += kThreads) {
+        for (int w = tid; w < m * m; w += nthr) {
             const int kk = w / m, ll = w % m;
             const int k = gidx[kk];
             const double* gk = W + L.gen + kGen * kk;
@@ -791,7 +1156,7 @@ dyn_kernel(DevNet net, EvalArgs a, OpfOut o, double damping_min, double* scratch
         if (kMode == DYN_FRONT) {                     // balanced FP32 matrix for the cluster kernel
             float* dst = hbuf + (size_t)s * hstride;
             float* A32 = dst + kHqHead;
-            for (int w = tid; w < n * n; w += kThreads) A32[w] = (float)A[w];
+            for (int w = tid; w < n * n; w += nthr) A32[w] = (float)A[w];
             if (tid == 0) dst[0] = __int_as_float(n);
             __syncthreads();
             balance<float>(A32, n, reinterpret_cast<float*>(cs_d), reinterpret_cast<float*>(rs_d), sh,
@@ -801,14 +1166,14 @@ dyn_kernel(DevNet net, EvalArgs a, OpfOut o, double damping_min, double* scratch
         }
         if (kMode == DYN_FRONT_LARGE) {               // balanced FP32 matrix, padded, for the tensor-core reduction
             float* A32 = reinterpret_cast<float*>(W + L.A32);
-            for (int w = tid; w < n * n; w += kThreads) A32[w] = (float)A[w];
+            for (int w = tid; w < n * n; w += nthr) A32[w] = (float)A[w];
             __syncthreads();
             balance<float>(A32, n, reinterpret_cast<float*>(cs_d), reinterpret_cast<float*>(rs_d), sh);
             __syncthreads();
             float* slot = hbuf + (size_t)s * hstride;
             const int nmax = 5 * ng - 1;
             float* M = slot + kHqHead;
-            for (int w = tid; w < nmax * nmax; w += kThreads) {
+            for (int w = tid; w < nmax * nmax; w += nthr) {
                 const int i = w / nmax, j = w % nmax;
                 M[w] = (i < n && j < n) ? A32[i * n + j] : (i == j ? -1.0f : 0.0f);
             }
@@ -818,10 +1183,10 @@ dyn_kernel(DevNet net, EvalArgs a, OpfOut o, double damping_min, double* scratch
         }
         if (kMode == DYN_MIXED_INLINE) {
             float* A32 = reinterpret_cast<float*>(W + L.A32);
-            for (int w = tid; w < n * n; w += kThreads) A32[w] = (float)A[w];
+            for (int w = tid; w < n * n; w += nthr) A32[w] = (float)A[w];
             __syncthreads();
             eigen_screen<float>(A32, n, reinterpret_cast<float*>(cs_d), reinterpret_cast<float*>(rs_d),
-                                reinterpret_cast<float*>(v_d), wr, wi, sh);
+                                reinterpret_cast<float*>(v_d), reinterpret_cast<float*>(W + L.hp), wr, wi, sh);
             eig_stats(sh, n, wr, wi, maxre, minz);
             const bool near = sh.fail || !(fabs(maxre) > kGuardRe) || !(fabs(minz - damping_min) > kGuardZeta);
             if (near) {                               // decision too close to call in FP32
@@ -830,11 +1195,11 @@ dyn_kernel(DevNet net, EvalArgs a, OpfOut o, double damping_min, double* scratch
                     atomicAdd(a.reruns, 1);
                 }
                 __syncthreads();
-                eigen_screen<double>(A, n, cs_d, rs_d, v_d, wr, wi, sh);
+                eigen_screen<double>(A, n, cs_d, rs_d, v_d, W + L.hp, wr, wi, sh);
                 eig_stats(sh, n, wr, wi, maxre, minz);
             }
         } else {
-            eigen_screen<double>(A, n, cs_d, rs_d, v_d, wr, wi, sh);
+            eigen_screen<double>(A, n, cs_d, rs_d, v_d, W + L.hp, wr, wi, sh);
             eig_stats(sh, n, wr, wi, maxre, minz);
         }
         // ---- 5. class ----
@@ -1078,13 +1443,14 @@ hqr_smem_kernel(EvalArgs a, OpfOut o, const float* __restrict__ hbuf, size_t hst
                 double damping_min, float* __restrict__ cand, int* counter) {
     extern __shared__ float qsm[];
     __shared__ float red[2][kQrThreads / 32];
-    __shared__ float xs[2][3];
+    __shared__ QrSpace<float> sp;
     __shared__ int scen;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     float* H = qsm;                                           // hq_off(nmax, nmax) floats
     int* rb = reinterpret_cast<int*>(qsm + ((hq_off(nmax, nmax) + 3) & ~3));   // row i at H[rb[i] + j]
     float* wr = reinterpret_cast<float*>(rb + nmax);
     float* wi = wr + nmax;
+    const PackedMat<float> A{H, rb};
     const float eps = 1.1920928955078125e-07f;
 
     for (;;) {
@@ -1164,83 +1530,8 @@ hqr_smem_kernel(EvalArgs a, OpfOut o, const float* __restrict__ hbuf, size_t hst
                 break;
             }
             ++its;
-            float sft, tft;
-            {
-                const float a11 = H[rb[hi - 1] + hi - 1], a12 = H[rb[hi - 1] + hi];
-                const float a21 = H[rb[hi] + hi - 1], a22 = H[rb[hi] + hi];
-                if (its % 10 == 0) {                       // exceptional shift, every tenth sweep
-                    const float ww = fabsf(a21) + fabsf(H[rb[hi - 1] + hi - 2]);
-                    sft = 1.5f * ww;
-                    tft = ww * ww;
-                } else {
-                    sft = a11 + a22;
-                    tft = a11 * a22 - a12 * a21;
-                }
-            }
-            float x0, x1, x2;
-            {
-                const float h00 = H[rb[lo] + lo], h01 = H[rb[lo] + lo + 1];
-                const float h10 = H[rb[lo + 1] + lo], h11 = H[rb[lo + 1] + lo + 1];
-                const float h21 = H[rb[lo + 2] + lo + 1];
-                x0 = h00 * h00 + h01 * h10 - sft * h00 + tft;
-                x1 = h10 * (h00 + h11 - sft);
-                x2 = h10 * h21;
-            }
-            __syncthreads();              // every warp has read the block and the shifts before the sweep writes
-            // rows this thread updates in the column phase (fixed for the sweep; the order is
-            // at most 2 * kQrThreads on this path), and their packed offsets
-            const int rbi0 = (lo + tid <= hi) ? rb[lo + tid] : 0;
-            const int rbi1 = (lo + tid + kQrThreads <= hi) ? rb[lo + tid + kQrThreads] : 0;
-            for (int k = lo; k <= hi - 1; ++k) {
-                const int len = (k + 2 <= hi) ? 3 : 2;
-                const float t2 = x1 * x1 + (len == 3 ? x2 * x2 : 0.0f);
-                const bool more = (k + 1 <= hi - 1);
-                if (t2 != 0.0f) {
-                    const float nrm = sqrtf(x0 * x0 + t2);
-                    const float al = (x0 >= 0.0f) ? -nrm : nrm;
-                    const float u0 = x0 - al, u1 = x1, u2 = (len == 3) ? x2 : 0.0f;
-                    const float bt = 2.0f / (u0 * u0 + t2);
-                    const int c0 = (k > lo) ? k - 1 : lo;
-                    const int b0 = rb[k], b1 = rb[k + 1], b2 = (len == 3) ? rb[k + 2] : 0;
-                    for (int j = c0 + tid; j <= hi; j += kQrThreads) {     // rows k..k+len-1
-                        const float p0 = H[b0 + j], p1 = H[b1 + j];
-                        const float p2 = (len == 3) ? H[b2 + j] : 0.0f;
-                        const float d = (u0 * p0 + u1 * p1 + u2 * p2) * bt;
-                        H[b0 + j] = p0 - d * u0;
-                        H[b1 + j] = p1 - d * u1;
-                        if (len == 3) H[b2 + j] = p2 - d * u2;
-                    }
-                    __syncthreads();
-                    const int r1 = (k + 3 < hi) ? k + 3 : hi;
-                    for (int i = lo + tid, m = 0; i <= r1; i += kQrThreads, ++m) {   // columns k..k+len-1
-                        float* p = H + (m == 0 ? rbi0 : rbi1) + k;
-                        const float q0 = p[0], q1 = p[1];
-                        const float q2 = (len == 3) ? p[2] : 0.0f;
-                        const float d = (q0 * u0 + q1 * u1 + q2 * u2) * bt;
-                        const float n0 = q0 - d * u0;
-                        p[0] = n0;
-                        p[1] = q1 - d * u1;
-                        if (len == 3) p[2] = q2 - d * u2;
-                        if (i > k && i <= k + 3) xs[k & 1][i - k - 1] = n0;     // next bulge column
-                    }
-                    __syncthreads();
-                    if (more) {
-                        x0 = xs[k & 1][0];
-                        x1 = xs[k & 1][1];
-                        x2 = (k + 3 <= hi) ? xs[k & 1][2] : 0.0f;
-                    }
-                } else if (more) {
-                    x0 = H[rb[k + 1] + k];
-                    x1 = H[rb[k + 2] + k];
-                    x2 = (k + 3 <= hi) ? H[rb[k + 3] + k] : 0.0f;
-                    __syncthreads();                       // all read before the next step writes column k
-                }
-            }
-            for (int i = lo + 2 + tid; i <= hi; i += kQrThreads) {
-                H[rb[i] + i - 2] = 0.0f;
-                if (i >= lo + 3) H[rb[i] + i - 3] = 0.0f;
-            }
-            __syncthreads();
+            __syncthreads();              // every warp has read the block before the sweep writes
+            qr_sweep<float>(A, lo, hi, its % 10 == 0, sp, kQrThreads, 0);  // exceptional shift every tenth sweep
         }
         __syncthreads();                                   // wr, wi written by thread 0
         // statistics over all eigenvalues: max Re, min damping ratio
@@ -1261,48 +1552,48 @@ hqr_smem_kernel(EvalArgs a, OpfOut o, const float* __restrict__ hbuf, size_t hst
             red[1][warp] = mz;
         }
         __syncthreads();
-        if (tid == 0) {
-            float maxre = red[0][0], minz = red[1][0];
-            for (int w = 1; w < kQrThreads / 32; ++w) {
-                maxre = fmaxf(maxre, red[0][w]);
-                minz = fminf(minz, red[1][w]);
-            }
+        if (warp == 0) {
+            float maxre = red[0][0];
+            for (int w = 1; w < kQrThreads / 32; ++w) maxre = fmaxf(maxre, red[0][w]);
             // The class is decided after the FP64 refinement (eig_refine_kernel), from
             // values within ~1e-9 of the FP64 screen's, so no FP32 guard band applies here;
             // a QR that did not converge goes to the FP64 screen.
-            if (fail) {
-                o.status[s] = 6;
-                atomicAdd(a.reruns, 1);
-            } else {
-                // Candidates of the FP64 refinement, in index order: every eigenvalue
-                // (im >= 0 of a pair) whose exact value may carry the largest real part
-                // or the smallest damping ratio, given |FP32 - exact| <= kEigDelta.
-                // Damping ratio of lambda with |delta lambda| <= d moves by at most 2 d / |lambda|.
-                float zu = INFINITY;
-                for (int i = 0; i < n; ++i) {
-                    if (wi[i] < 0.0f) continue;
-                    const float mg = sqrtf(wr[i] * wr[i] + wi[i] * wi[i]);
-                    const float z = mg > 0.0f ? -wr[i] / mg : 1.0f;
-                    zu = fminf(zu, mg > 0.0f ? z + 2.0f * kEigDelta / mg : INFINITY);
+            // Candidates of the FP64 refinement, in index order: every eigenvalue
+            // (im >= 0 of a pair) whose exact value may carry the largest real part
+            // or the smallest damping ratio, given |FP32 - exact| <= kEigDelta.
+            // Damping ratio of lambda with |delta lambda| <= d moves by at most 2 d / |lambda|.
+            auto modulus = [&](int i) { return sqrtf(wr[i] * wr[i] + wi[i] * wi[i]); };
+            float zu = INFINITY;
+            if (!fail)
+                for (int i = lane; i < n; i += 32) {
+                    const float mg = modulus(i);
+                    if (!(wi[i] < 0.0f) && mg > 0.0f) zu = fminf(zu, -wr[i] / mg + 2.0f * kEigDelta / mg);
                 }
-                float* cs = cand + (size_t)s * kCandStride;
-                int cnt = 0, flags = 0;
-                for (int i = 0; i < n; ++i) {
-                    if (wi[i] < 0.0f) continue;
-                    const float mg = sqrtf(wr[i] * wr[i] + wi[i] * wi[i]);
+            for (int off = 16; off; off >>= 1) zu = fminf(zu, __shfl_xor_sync(0xffffffffu, zu, off));
+            float* cs = cand + (size_t)s * kCandStride;
+            int cnt = 0, flags = 0;
+            for (int i0 = 0; i0 < n && !fail; i0 += 32) {
+                const int i = i0 + lane;
+                bool cre = false, cz = false;
+                if (i < n && !(wi[i] < 0.0f)) {
+                    const float mg = modulus(i);
                     const float z = mg > 0.0f ? -wr[i] / mg : 1.0f;
-                    const bool cre = wr[i] >= maxre - 2.0f * kEigDelta;
-                    const bool cz = !(mg > 0.0f) || z - 2.0f * kEigDelta / mg <= zu;
-                    if (!cre && !cz) continue;
-                    if (cnt < kRefK) {
+                    cre = wr[i] >= maxre - 2.0f * kEigDelta;
+                    cz = !(mg > 0.0f) || z - 2.0f * kEigDelta / mg <= zu;
+                }
+                for (unsigned m = __ballot_sync(0xffffffffu, cre || cz); m; m &= m - 1, ++cnt) {
+                    const int src = __ffs(m) - 1;
+                    const int f = __shfl_sync(0xffffffffu, (cre ? 1 : 0) | (cz ? 2 : 0), src);
+                    if (cnt >= kRefK) continue;
+                    flags |= f << (2 * cnt);
+                    if (lane == src) {
                         cs[4 + 2 * cnt] = wr[i];
                         cs[5 + 2 * cnt] = wi[i];
-                        flags |= (cre ? 1 : 0) << (2 * cnt);
-                        flags |= (cz ? 2 : 0) << (2 * cnt);
                     }
-                    ++cnt;
                 }
-                if (cnt > kRefK) {                         // too many to refine: FP64 screen
+            }
+            if (lane == 0) {
+                if (fail || cnt > kRefK) {                 // not converged, or too many to refine: FP64 screen
                     o.status[s] = 6;
                     atomicAdd(a.reruns, 1);
                 } else {
@@ -1647,6 +1938,8 @@ eig_refine_kernel(EvalArgs a, OpfOut o, const float* __restrict__ hbuf, size_t h
 
 }  // namespace
 
+int dyn_ctas_per_sm() { return kCtasPerSm; }
+
 size_t dyn_scratch_doubles(const DevNet& net) { return (size_t)make_dlayout(net).total; }
 
 size_t dyn_hbuf_stride(const DevNet& net) {
@@ -1690,14 +1983,20 @@ bool dyn_split_fits(const DevNet& net, int device) {
 template <int kMode>
 static cudaError_t launch_mode(const DevNet& net, const EvalArgs& a, OpfOut o, double damping_min, double* scratch,
                                size_t per_cta, const DLay& L, float* hbuf, size_t hstride, double* a64, int grid,
-                               int* counter, cudaStream_t s) {
+                               int sms, int* counter, cudaStream_t s) {
     const size_t smem = sizeof(double) * ((size_t)((net.ng + 1) >> 1) + 15 * (size_t)net.ng);
     if (smem > 48 * 1024) {
         cudaError_t e = cudaFuncSetAttribute(dyn_kernel<kMode>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
     }
-    dyn_kernel<kMode><<<grid, kThreads, smem, s>>>(net, a, o, damping_min, scratch, per_cta, L, hbuf, hstride, a64,
-                                                   dyn_a64_stride(net), counter);
+    // One block has a chain of dependent FP64 steps (the QR bulge, one warp) between wide phases: with
+    // few scenarios a block of many threads shortens the wide phases, with many scenarios small blocks,
+    // four per SM, fill one another's chains.  Results do not depend on the number of threads.
+    // 118 buses, FP64 screen: 2,000 pairs 572 ms with four blocks of 128 threads per SM, 713 with two of 256
+    // (510 now, with the one-pass Hessenberg reduction); 240 single outages 144 and 124 (114 now).
+    const int threads = grid > 2 * sms ? 128 : grid > sms ? 256 : 512;
+    dyn_kernel<kMode><<<grid, threads, smem, s>>>(net, a, o, damping_min, scratch, per_cta, L, hbuf, hstride, a64,
+                                                  dyn_a64_stride(net), counter);
     return cudaGetLastError();
 }
 
@@ -1715,7 +2014,7 @@ cudaError_t launch_dyn(const DevNet& net, const EvalArgs& a, OpfOut o, double da
         // SM, FP64 refinement of the decisive eigenvalues, and the FP64 re-run of the
         // scenarios the FP32 screen cannot decide.
         const size_t hstride = dyn_hbuf_stride(net), astride = dyn_abuf_stride(net);
-        e = launch_mode<DYN_FRONT>(net, a, o, damping_min, scratch, scratch_per_cta, L, abuf, astride, a64, grid,
+        e = launch_mode<DYN_FRONT>(net, a, o, damping_min, scratch, scratch_per_cta, L, abuf, astride, a64, grid, sms,
                                    counters, s);
         if (e != cudaSuccess) return e;
         const int nmax = 5 * net.ng - 1;
@@ -1740,7 +2039,7 @@ cudaError_t launch_dyn(const DevNet& net, const EvalArgs& a, OpfOut o, double da
                                                        cand, nmax, damping_min, counters + 4);
         e = cudaGetLastError();
         if (e != cudaSuccess) return e;
-        e = launch_mode<DYN_RERUN>(net, a, o, damping_min, scratch, scratch_per_cta, L, nullptr, 0, nullptr, grid,
+        e = launch_mode<DYN_RERUN>(net, a, o, damping_min, scratch, scratch_per_cta, L, nullptr, 0, nullptr, grid, sms,
                                    counters + 2, s);
         if (e != cudaSuccess) return e;
         *launches = 5;
@@ -1750,25 +2049,23 @@ cudaError_t launch_dyn(const DevNet& net, const EvalArgs& a, OpfOut o, double da
         // cores, FP32 QR per scenario, FP64 re-run of the undecided ones
         const int nmax = 5 * net.ng - 1;
         const size_t astride = dyn_abuf_stride(net);
-        e = launch_mode<DYN_FRONT_LARGE>(net, a, o, damping_min, scratch, scratch_per_cta, L, abuf, astride, nullptr,
-                                         grid, counters, s);
+        e = launch_mode<DYN_FRONT_LARGE>(net, a, o, damping_min, scratch, scratch_per_cta, L, abuf, astride, nullptr, grid, sms, counters, s);
         if (e != cudaSuccess) return e;
         e = launch_hess_tc(a.n, nmax, abuf + kHqHead, (long long)astride, hws, a.err, s);
         if (e != cudaSuccess) return e;
-        e = launch_mode<DYN_QR_LARGE>(net, a, o, damping_min, scratch, scratch_per_cta, L, abuf, astride, nullptr, grid,
+        e = launch_mode<DYN_QR_LARGE>(net, a, o, damping_min, scratch, scratch_per_cta, L, abuf, astride, nullptr, grid, sms,
                                       counters + 1, s);
         if (e != cudaSuccess) return e;
-        e = launch_mode<DYN_RERUN>(net, a, o, damping_min, scratch, scratch_per_cta, L, nullptr, 0, nullptr, grid,
+        e = launch_mode<DYN_RERUN>(net, a, o, damping_min, scratch, scratch_per_cta, L, nullptr, 0, nullptr, grid, sms,
                                    counters + 2, s);
         if (e != cudaSuccess) return e;
         *launches = 4;
     } else if (precision == CS_PREC_MIXED) {
-        e = launch_mode<DYN_MIXED_INLINE>(net, a, o, damping_min, scratch, scratch_per_cta, L, nullptr, 0, nullptr,
-                                          grid, counters, s);
+        e = launch_mode<DYN_MIXED_INLINE>(net, a, o, damping_min, scratch, scratch_per_cta, L, nullptr, 0, nullptr, grid, sms, counters, s);
         if (e != cudaSuccess) return e;
         *launches = 1;
     } else {
-        e = launch_mode<DYN_FULL64>(net, a, o, damping_min, scratch, scratch_per_cta, L, nullptr, 0, nullptr, grid,
+        e = launch_mode<DYN_FULL64>(net, a, o, damping_min, scratch, scratch_per_cta, L, nullptr, 0, nullptr, grid, sms,
                                     counters, s);
         if (e != cudaSuccess) return e;
         *launches = 1;
