@@ -100,8 +100,6 @@ struct DShared {
     int ired[kMaxThreads / 32];
     double hs[3];                    // Hessenberg reduction: tail, alpha, beta of the current column
     int fail, scen, m, nn;
-    double bal_f;
-    int bal_i;
 };
 
 // block reductions ---------------------------------------------------------
@@ -155,26 +153,51 @@ __device__ void eig2(double p, double q, double r, double s, double* re, double*
 // Balancing (radix 2).  Each sweep starts from exact off-diagonal column and
 // row 1-norms; within the sweep the norms are updated as rows and columns are
 // scaled (a scaling by a power of two changes the other norms by a known
-// amount), so the sequential scan over the indices needs no reduction.  One
-// thread takes each index's decision; only indices that are scaled cost a
-// pass over the matrix.  The scale search stops at 2^+-kBalExp (T = float) or
+// amount), so the scan over the indices needs no reduction: all threads look at
+// their indices' norms at once, and the first one that wants a factor is scaled.
+// The sequential sweeps end it as they always did (until no index improves by
+// 5 %), but most factors come from kBalJoint sweeps before them that scale all
+// indices at once, each by the root of its best factor: an entry joins two
+// indices, and with both moved the whole way it would overshoot.  (A factor of
+// 2 has no root here: the two halves of the indices take those in turn.)  One
+// index at a time costs two barriers and two strided passes; a joint sweep two
+// passes over the matrix.
+// (118 buses, front kernel: one scenario 2.0 -> 1.3 ms, 417 of them 5.2 -> 4.8.)
+// The scale search stops at 2^+-kBalExp (T = float) or
 // 2^+-(4 kBalExp) (T = double), so a row or column norm that is tiny next to
 // the other cannot drive the factor to overflow or zero; an index whose best
-// factor lies beyond that is scaled by the bound.  When dsc is given, dsc[i]
+// factor lies beyond that is scaled by the bound.  dsc[i]
 // receives the product of the factors of index i: the balanced matrix is
 // diag(dsc)^-1 A diag(dsc), exactly (every factor is a power of two).
 constexpr int kBalExp = 30;
+constexpr int kBalJoint = 12;
+
+// exponent of the factor of an index with column norm c and row norm r; 0: leave it
 template <typename T>
-__device__ void balance(T* A, const int n, T* cs, T* rs, DShared& sh, T* dsc = nullptr) {
+__device__ __forceinline__ int bal_exponent(T c, const T r) {
+    if (c == 0 || r == 0 || !isfinite(c) || !isfinite(r)) return 0;
+    constexpr int top = sizeof(T) == 8 ? 4 * kBalExp : kBalExp;
+    const T ssum = c + r;
+    T g = r / 2, f = 1;
+    int e = 0;
+    while (c < g && e < top) { f *= 2; c *= 4; ++e; }
+    g = r * 2;
+    while (c > g && e > -top) { f /= 2; c /= 4; --e; }
+    return ((c + r) / f < (T)0.95 * ssum) ? e : 0;
+}
+
+template <typename T>
+__device__ void balance(T* A, const int n, T* cs, T* rs, T* dsc, DShared& sh) {
     const int tid = threadIdx.x, nthr = blockDim.x, warp = tid >> 5, lane = tid & 31;
-    const T fmaxb = (T)ldexp(1.0, sizeof(T) == 8 ? 4 * kBalExp : kBalExp), fminb = (T)1 / fmaxb;
-    if (dsc)
-        for (int j = tid; j < n; j += nthr) dsc[j] = (T)1;
-    for (int sweep = 0; sweep < 100; ++sweep) {
+    for (int j = tid; j < n; j += nthr) dsc[j] = (T)1;
+    for (int sweep = 0; sweep < kBalJoint + 100; ++sweep) {
         for (int j = tid; j < n; j += nthr) {
             T c = 0;
-            for (int i = 0; i < n; ++i)
-                if (i != j) c += fabs(A[(size_t)i * n + j]);
+#pragma unroll 8
+            for (int i = 0; i < n; ++i) {
+                const T a = fabs(A[(size_t)i * n + j]);
+                c += (i != j) ? a : (T)0;
+            }
             cs[j] = c;
         }
         for (int i = warp; i < n; i += nthr / 32) {
@@ -185,35 +208,44 @@ __device__ void balance(T* A, const int n, T* cs, T* rs, DShared& sh, T* dsc = n
             if (lane == 0) rs[i] = r;
         }
         __syncthreads();
+        if (sweep < kBalJoint) {
+            int any = 0;
+            for (int i = tid; i < n; i += nthr) {
+                int e = bal_exponent(cs[i], rs[i]);
+                if (e == 1 || e == -1) e = ((i ^ sweep) & 1) ? 0 : e;
+                else e /= 2;
+                any |= e;
+                cs[i] = ldexp((T)1, e);                        // the norms have been read: now the factors
+                dsc[i] *= cs[i];
+            }
+            any = __syncthreads_or(any);
+            if (any == 0) {
+                sweep = kBalJoint - 1;
+                continue;
+            }
+            for (int i = warp; i < n; i += nthr / 32) {
+                const T fi = (T)1 / cs[i];
+                for (int j = lane; j < n; j += 32) A[(size_t)i * n + j] *= fi * cs[j];
+            }
+            __syncthreads();
+            continue;
+        }
         bool changed = false;
         int i0 = 0;
         for (;;) {
-            if (tid == 0) {
-                int pick = -1;
-                double fpick = 1.0;
-                for (int i = i0; i < n && pick < 0; ++i) {
-                    T c = cs[i];
-                    const T r = rs[i];
-                    if (c == 0 || r == 0 || !isfinite(c) || !isfinite(r)) continue;
-                    T g = r / 2, f = 1;
-                    const T ssum = c + r;
-                    while (c < g && f < fmaxb) { f *= 2; c *= 4; }
-                    g = r * 2;
-                    while (c > g && f > fminb) { f /= 2; c /= 4; }
-                    if ((c + r) / f < (T)0.95 * ssum) { pick = i; fpick = (double)f; }
-                }
-                sh.bal_i = pick;
-                sh.bal_f = fpick;
-            }
-            __syncthreads();
-            const int i = sh.bal_i;
-            if (i < 0) break;
-            const T f = (T)sh.bal_f, finv = (T)(1.0 / sh.bal_f);
+            int pick = n;
+            for (int i = i0 + tid; i < n && pick == n; i += nthr)
+                if (bal_exponent(cs[i], rs[i]) != 0) pick = i;
+            const int i = -bmax_int(sh, -pick);
+            if (i >= n) break;
+            const int e = bal_exponent(cs[i], rs[i]);
+            const T f = ldexp((T)1, e), finv = ldexp((T)1, -e);
+            __syncthreads();                                   // cs[i], rs[i] read by all
             for (int j = tid; j < n; j += nthr) {
                 if (j == i) {
                     cs[i] *= f;
                     rs[i] *= finv;
-                    if (dsc) dsc[i] *= f;
+                    dsc[i] *= f;
                     continue;
                 }
                 const T a = A[(size_t)i * n + j], b = A[(size_t)j * n + i];
@@ -390,30 +422,33 @@ struct alignas(16) QrStep {                      // reflector of one step
     T v1, v2, tau;
 };
 template <typename T>
-struct QrSpace;                                  // in shared memory
-template <>
-struct QrSpace<double> {
-    QrStep<double> st[kQrNB<double>];
-};
-template <>
-struct QrSpace<float> {
-    QrStep<float> st[kQrNB<float>];
-    float blk[kQrNB<float> + 3][kQrNB<float> + 3];             // the window's first columns (odd row stride)
+struct QrSpace {                                 // in shared memory
+    QrStep<T> st[kQrNB<T>];
 };
 
-// 1 / sqrt(x) and 1 / x: the hardware approximations in FP32 (2 units in the last place; the
-// reflector's departure from orthogonality stays at rounding level).  In FP64 the FP32 approximation
-// and one step of Halley's iteration (third order: 2^-22 -> 2^-66 relative before rounding), five and
-// three FP64 instructions.  Arguments within 1e-30 .. 1e30.
-__device__ __forceinline__ float qr_rsqrt(float x) {
+// 1 / sqrt(x) and 1 / x.  FP32: the hardware approximation and one Newton step, to rounding level: a
+// reflector that is orthogonal to 2^-22 only, with the approximation's bias, moves the eigenvalues by
+// more than the refinement allows for after the few hundred sweeps (one to three scenarios of 24,000
+// went to the FP64 screen for it).  FP64: the FP32 approximation and one step of Halley's
+// iteration (third order: 2^-22 -> 2^-66 relative before rounding), five and three FP64
+// instructions.  Arguments within 1e-30 .. 1e30.
+__device__ __forceinline__ float rsqrt_approx(float x) {
     float r;
     asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
     return r;
 }
-__device__ __forceinline__ float qr_rcp(float x) {
+__device__ __forceinline__ float rcp_approx(float x) {
     float r;
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
     return r;
+}
+__device__ __forceinline__ float qr_rsqrt(float x) {
+    const float y = rsqrt_approx(x), e = fmaf(-(x * y), y, 1.0f);
+    return fmaf(0.5f * y, e, y);
+}
+__device__ __forceinline__ float qr_rcp(float x) {
+    const float y = rcp_approx(x);
+    return fmaf(y, fmaf(-x, y, 1.0f), y);
 }
 // (The seeds' conversions run on the integer pipe: an FP64 conversion costs an FP64 instruction.)
 __device__ __forceinline__ float qr_seed(double x) {        // x truncated to FP32
@@ -425,11 +460,11 @@ __device__ __forceinline__ double qr_wide(float y) {
     return __hiloint2double((b >> 3) + (896 << 20), b << 29);
 }
 __device__ __forceinline__ double qr_rsqrt(double x) {
-    const double y = qr_wide(qr_rsqrt(qr_seed(x))), e = fma(-(x * y), y, 1.0);
+    const double y = qr_wide(rsqrt_approx(qr_seed(x))), e = fma(-(x * y), y, 1.0);
     return fma(y * e, fma(0.375, e, 0.5), y);
 }
 __device__ __forceinline__ double qr_rcp(double x) {
-    const double y = qr_wide(qr_rcp(qr_seed(x))), e = fma(-x, y, 1.0);
+    const double y = qr_wide(rcp_approx(qr_seed(x))), e = fma(-x, y, 1.0);
     return fma(y, fma(e, e, e), y);
 }
 // x within about 1e-30 .. 1e30 (x a sum of squares: not negative; NaN and infinity are not)
@@ -510,144 +545,96 @@ __device__ __forceinline__ void qr_apply(T (&y)[kQrNB<T> + 2], const QrSpace<T>&
     }
 }
 
-// Steps kw .. kw + cnt - 1 of the sweep, one warp, the bulge in and out.  Two forms.
+// Steps kw .. kw + cnt - 1 of the sweep, one warp, the bulge in and out.  The right reflectors are
+// applied to the three rows below the bulge at once, as the next reflector needs; the window's rows
+// take the rest of them in the strips, each from its own step on.  So every entry takes its
+// reflections in the order of the step-by-step sweep.  (All left reflectors first and the right ones
+// after them is the same product and a shorter step, but the entries below the bulge then come
+// from cancellation within the window: in FP32 one to three scenarios of 24,000 did not converge.)
 //
-// FP64: the right reflectors are applied to the three rows below the bulge in the lanes too; the
-// nine entries they need are fetched by shuffles, which take less time than an FP64 instruction.
-// The window's rows take the rest of the right reflectors in the strips, each from its own step on.
-template <bool kFull, typename M>
-__device__ __forceinline__ void qr_chase(const M& A, int lo, int hi, int kw, int cnt, QrBulge<double>& bu,
-                                         QrSpace<double>& sp) {
+// In FP32 the chain from one reflector to the next runs on copies of its few entries that every
+// lane keeps: rows k .. k + 2 of columns k and k + 1, and column k + 2, fetched before the reflector
+// is known.  An FP64 instruction takes longer than a shuffle, so there the entries are fetched.
+template <bool kFull, typename T, typename M>
+__device__ __forceinline__ void qr_chase(const M& A, int lo, int hi, int kw, int cnt, QrBulge<T>& bu, QrSpace<T>& sp) {
+    constexpr int NB = kQrNB<T>;
+    constexpr bool kCopies = sizeof(T) == 4;
     const unsigned all = 0xffffffffu;
     const int lane = threadIdx.x & 31, col = kw + lane;
-    double w[kQrNB<double> + 3];
+    T w[NB + 3];
 #pragma unroll
-    for (int r = 0; r < kQrNB<double> + 3; ++r)
-        w[r] = ((kFull || (kw + r <= hi)) && col <= hi && lane + 1 >= r) ? *A.at(kw + r, col) : 0.0;
+    for (int r = 0; r < NB + 3; ++r)
+        w[r] = ((kFull || kw + r <= hi) && col <= hi && lane + 1 >= r) ? *A.at(kw + r, col) : (T)0;
     if (lane == 0) w[2] = bu.b;
-    double x0 = bu.x0, x1 = bu.x1, x2 = bu.x2, sub = 0;   // sub: subdiagonal entry (kw + lane, kw + lane - 1)
+    T x0 = bu.x0, x1 = bu.x1, x2 = bu.x2, sub = 0;        // sub: subdiagonal entry (kw + lane, kw + lane - 1)
+    T m00 = 0, m01 = 0, m10 = 0, m11 = 0, m20 = 0, m21 = 0;
+    if (kCopies) {
+        m00 = __shfl_sync(all, w[0], 0); m01 = __shfl_sync(all, w[0], 1);
+        m10 = __shfl_sync(all, w[1], 0); m11 = __shfl_sync(all, w[1], 1);
+        m20 = bu.b;                      m21 = __shfl_sync(all, w[2], 1);
+    }
 #pragma unroll
-    for (int t = 0; t < kQrNB<double>; ++t) {
+    for (int t = 0; t < NB; ++t) {
         if (!kFull && t >= cnt) break;
-        const QrRefl<double> h = qr_reflector(x0, x1, x2);
-        const double v1 = h.v1, v2 = h.v2, tau = h.tau, t1 = tau * v1, t2 = tau * v2;
-        if (lane == t) {
-            sub = h.alpha;
-            sp.st[t] = {v1, v2, tau};
+        T c0 = 0, c1 = 0, c2 = 0, s3 = 0;
+        if (kCopies) {
+            c0 = __shfl_sync(all, w[t], t + 2);
+            c1 = __shfl_sync(all, w[t + 1], t + 2);
+            c2 = __shfl_sync(all, w[t + 2], t + 2);
+            s3 = __shfl_sync(all, w[t + 3], t + 2);
         }
-        const double d = w[t] + v1 * w[t + 1] + v2 * w[t + 2];   // left, rows kw + t ..
+        const QrRefl<T> h = qr_reflector(x0, x1, x2);
+        const T v1 = h.v1, v2 = h.v2, tau = h.tau, t1 = tau * v1, t2 = tau * v2;
+        sp.st[t] = {v1, v2, tau};                         // the same from every lane
+        if (lane == t) sub = h.alpha;
+        T da, db, dc;
+        if (kCopies) {
+            const T d0 = m00 + v1 * m10 + v2 * m20, d1 = m01 + v1 * m11 + v2 * m21, d2 = c0 + v1 * c1 + v2 * c2;
+            const T n10 = m10 - t1 * d0, n20 = m20 - t2 * d0, n11 = m11 - t1 * d1, n21 = m21 - t2 * d1,
+                    n12 = c1 - t1 * d2, n22 = c2 - t2 * d2;
+            da = n10 + v1 * n11 + v2 * n12;
+            db = n20 + v1 * n21 + v2 * n22;
+            dc = v2 * s3;
+            x0 = n10 - tau * da;
+            x1 = n20 - tau * db;
+            x2 = -(tau * dc);
+            m00 = n11 - t1 * da; m01 = n12 - t2 * da;
+            m10 = n21 - t1 * db; m11 = n22 - t2 * db;
+            m20 = -(t1 * dc);    m21 = s3 - t2 * dc;
+        }
+        const T d = w[t] + v1 * w[t + 1] + v2 * w[t + 2]; // left, rows kw + t ..
         w[t] -= tau * d;
         w[t + 1] -= t1 * d;
         w[t + 2] -= t2 * d;
-        const double a0 = __shfl_sync(all, w[t + 1], t), a1 = __shfl_sync(all, w[t + 1], t + 1),
-                     a2 = __shfl_sync(all, w[t + 1], t + 2);
-        const double b0 = __shfl_sync(all, w[t + 2], t), b1 = __shfl_sync(all, w[t + 2], t + 1),
-                     b2 = __shfl_sync(all, w[t + 2], t + 2);
-        const double da = a0 + v1 * a1 + v2 * a2, db = b0 + v1 * b1 + v2 * b2, dc = v2 * __shfl_sync(all, w[t + 3], t + 2);
-        const double co = lane == t ? tau : lane == t + 1 ? t1 : lane == t + 2 ? t2 : 0.0;
+        if (!kCopies) {                                   // right, the three rows below
+            const T a0 = __shfl_sync(all, w[t + 1], t), a1 = __shfl_sync(all, w[t + 1], t + 1),
+                    a2 = __shfl_sync(all, w[t + 1], t + 2);
+            const T b0 = __shfl_sync(all, w[t + 2], t), b1 = __shfl_sync(all, w[t + 2], t + 1),
+                    b2 = __shfl_sync(all, w[t + 2], t + 2);
+            da = a0 + v1 * a1 + v2 * a2;
+            db = b0 + v1 * b1 + v2 * b2;
+            dc = v2 * __shfl_sync(all, w[t + 3], t + 2);
+        }
+        // (column kw + t itself is the next bulge column: only needed as x)
+        const T co = lane == t + 1 ? t1 : lane == t + 2 ? t2 : kCopies ? (T)0 : lane == t ? tau : (T)0;
         w[t + 1] -= co * da;
         w[t + 2] -= co * db;
         w[t + 3] -= co * dc;
-        x0 = __shfl_sync(all, w[t + 1], t);
-        x1 = __shfl_sync(all, w[t + 2], t);
-        x2 = __shfl_sync(all, w[t + 3], t);
+        if (!kCopies) {
+            x0 = __shfl_sync(all, w[t + 1], t);
+            x1 = __shfl_sync(all, w[t + 2], t);
+            x2 = __shfl_sync(all, w[t + 3], t);
+        }
     }
-    bu = QrBulge<double>{x0, x1, x2, kFull ? __shfl_sync(all, w[kQrNB<double> + 2], kQrNB<double>) : 0.0};
+    bu = QrBulge<T>{x0, x1, x2, kCopies ? m20 : kFull ? __shfl_sync(all, w[NB + 2], NB) : (T)0};
     // a column of the window is final on and above its diagonal; its subdiagonal entry is the next
     // step's alpha (the last one's, the next window's, or x0 at the end of the sweep)
 #pragma unroll
-    for (int r = 0; r < kQrNB<double> + 3; ++r)
+    for (int r = 0; r < NB + 3; ++r)
         if ((kFull || kw + r <= hi) && col <= hi && (lane >= r || (lane + 1 == r && lane >= cnt)))
             *A.at(kw + r, col) = w[r];
     if (lane < cnt && col > lo) *A.at(col, col - 1) = sub;
     if (kw + cnt == hi && lane == 0) *A.at(hi, hi - 1) = x0;
-}
-
-// FP32: the lanes take the left reflectors only (left and right ones commute), and the chain from one
-// reflector to the next runs on copies of its few entries that every lane keeps: rows k .. k + 2 of
-// columns k and k + 1, and column k + 2, fetched before the reflector is known.  So no shuffle lies on
-// the chain and a step is ~50 instructions of one warp.  The right reflectors act on the window's
-// first columns in the strips (sp.blk holds them meanwhile, with the entries that the left reflectors
-// fill below the subdiagonal).
-template <bool kFull, typename M>
-__device__ __forceinline__ void qr_chase(const M& A, int lo, int hi, int kw, int cnt, QrBulge<float>& bu,
-                                         QrSpace<float>& sp) {
-    const unsigned all = 0xffffffffu;
-    const int lane = threadIdx.x & 31, col = kw + lane;
-    float w[kQrNB<float> + 3];
-#pragma unroll
-    for (int r = 0; r < kQrNB<float> + 3; ++r)
-        w[r] = ((kFull || (kw + r <= hi)) && col <= hi && lane + 1 >= r) ? *A.at(kw + r, col) : 0.0f;
-    if (lane == 0) w[2] = bu.b;
-    float x0 = bu.x0, x1 = bu.x1, x2 = bu.x2, sub = 0;    // sub: subdiagonal entry (kw + lane, kw + lane - 1)
-    float m00 = __shfl_sync(all, w[0], 0), m01 = __shfl_sync(all, w[0], 1);
-    float m10 = __shfl_sync(all, w[1], 0), m11 = __shfl_sync(all, w[1], 1);
-    float m20 = bu.b, m21 = __shfl_sync(all, w[2], 1);
-#pragma unroll
-    for (int t = 0; t < kQrNB<float>; ++t) {
-        if (!kFull && t >= cnt) break;
-        const float c0 = __shfl_sync(all, w[t], t + 2), c1 = __shfl_sync(all, w[t + 1], t + 2),
-                    c2 = __shfl_sync(all, w[t + 2], t + 2), s3 = __shfl_sync(all, w[t + 3], t + 2);
-        const QrRefl<float> h = qr_reflector(x0, x1, x2);
-        const float v1 = h.v1, v2 = h.v2, tau = h.tau, t1 = tau * v1, t2 = tau * v2;
-        sp.st[t] = {v1, v2, tau};                         // the same from every lane
-        if (lane == t) sub = h.alpha;
-        const float d0 = m00 + v1 * m10 + v2 * m20, d1 = m01 + v1 * m11 + v2 * m21, d2 = c0 + v1 * c1 + v2 * c2;
-        const float n10 = m10 - t1 * d0, n20 = m20 - t2 * d0, n11 = m11 - t1 * d1, n21 = m21 - t2 * d1,
-                    n12 = c1 - t1 * d2, n22 = c2 - t2 * d2;
-        const float da = n10 + v1 * n11 + v2 * n12, db = n20 + v1 * n21 + v2 * n22, dc = v2 * s3;
-        x0 = n10 - tau * da;
-        x1 = n20 - tau * db;
-        x2 = -(tau * dc);
-        m00 = n11 - t1 * da; m01 = n12 - t2 * da;
-        m10 = n21 - t1 * db; m11 = n22 - t2 * db;
-        m20 = -(t1 * dc);    m21 = s3 - t2 * dc;
-        const float d = w[t] + v1 * w[t + 1] + v2 * w[t + 2];     // left, rows kw + t ..
-        w[t] -= tau * d;
-        w[t + 1] -= t1 * d;
-        w[t + 2] -= t2 * d;
-    }
-    bu = QrBulge<float>{x0, x1, x2, m20};
-    if (lane < kQrNB<float> + 2) {
-#pragma unroll
-        for (int r = 0; r < kQrNB<float> + 3; ++r) sp.blk[r][lane] = w[r];
-    } else if (col <= hi) {                               // right of the reflectors' columns: final
-#pragma unroll
-        for (int r = 0; r < kQrNB<float> + 3; ++r)
-            if ((kFull || kw + r <= hi) && lane + 1 >= r) *A.at(kw + r, col) = w[r];
-    }
-    if (lane < cnt && col > lo) *A.at(col, col - 1) = sub;
-    if (kw + cnt == hi && lane == 0) *A.at(hi, hi - 1) = x0;
-}
-
-// The window's own rows in the strips: FP64, from the matrix, each row from its own step on; FP32, from
-// sp.blk, all of them.
-template <typename M>
-__device__ __forceinline__ void qr_own_rows(const M& A, int hi, int kw, int cnt, const QrSpace<double>& sp, int lane) {
-    if (lane >= cnt) return;
-    double y[kQrNB<double> + 2];
-    double* row = A.at(kw + lane, kw);
-#pragma unroll
-    for (int c = 0; c < kQrNB<double> + 2; ++c) y[c] = (c >= lane && c <= cnt + 1 && kw + c <= hi) ? row[c] : 0.0;
-    qr_apply<false>(y, sp, lane, cnt);
-#pragma unroll
-    for (int c = 0; c < kQrNB<double> + 2; ++c)
-        if (c >= lane && c <= cnt + 1 && kw + c <= hi) row[c] = y[c];
-}
-template <typename M>
-__device__ __forceinline__ void qr_own_rows(const M& A, int hi, int kw, int cnt, const QrSpace<float>& sp, int lane) {
-    if (lane >= kQrNB<float> + 3 || kw + lane > hi) return;
-    float y[kQrNB<float> + 2];
-#pragma unroll
-    for (int c = 0; c < kQrNB<float> + 2; ++c) y[c] = sp.blk[lane][c];
-    if (cnt == kQrNB<float>) qr_apply<true>(y, sp, 0, kQrNB<float>);
-    else qr_apply<false>(y, sp, 0, cnt);
-    float* row = A.at(kw + lane, kw);
-    // on and right of the diagonal; below it only the entries right of the bulge column (the
-    // others are the steps' alphas and zeros)
-#pragma unroll
-    for (int c = 0; c < kQrNB<float> + 2; ++c)
-        if (kw + c <= hi && (c >= lane || (c + 1 == lane && c >= cnt))) row[c] = y[c];
 }
 
 // The window's reflectors on the rows above it, the columns right of it, and its own rows (each from
@@ -687,26 +674,37 @@ __device__ __forceinline__ void qr_strips(const M& A, int lo, int hi, int kw, in
 #pragma unroll
             for (int r = 0; r < kQrNB<T> + 2; ++r) *A.at(kw + r, j) = y[r];
         } else {
-            qr_own_rows(A, hi, kw, cnt, sp, lane);
+            if (lane >= cnt) continue;
+            T* row = A.at(kw + lane, kw);
+#pragma unroll
+            for (int c = 0; c < kQrNB<T> + 2; ++c) y[c] = (c >= lane && c <= cnt + 1 && kw + c <= hi) ? row[c] : (T)0;
+            qr_apply<false>(y, sp, lane, cnt);
+#pragma unroll
+            for (int c = 0; c < kQrNB<T> + 2; ++c)
+                if (c >= lane && c <= cnt + 1 && kw + c <= hi) row[c] = y[c];
         }
     }
 }
 
-// First column of the double-shift step: (H^2 - s H + t I) e1 of the block lo..hi, with the shifts'
-// sum s and product t from its trailing 2x2 block or, if exceptional, from its last subdiagonals.
+// First column of the double-shift step, (H - a I)(H - b I) e1 / h10 of the block lo..hi, a and b the
+// eigenvalues of its trailing 2x2 block (or, if exceptional, a pair off its last entry by the size of
+// the last subdiagonals), in differences to the leading diagonal entry: formed from the shifts' sum
+// and product, a block whose eigenvalues differ by little (the exciters' cluster near -1/T_A) loses
+// the differences to cancellation in FP32 and its sweeps go nowhere (118 buses: 331 -> 276 sweeps a
+// scenario, and the scenario in 20,000 that ran to the sweep limit converges).
 template <typename T, typename M>
 __device__ __forceinline__ void qr_start(const M& A, int lo, int hi, bool exceptional, QrBulge<T>& bu) {
-    const T a11 = *A.at(hi - 1, hi - 1), a12 = *A.at(hi - 1, hi), a21 = *A.at(hi, hi - 1), a22 = *A.at(hi, hi);
-    T sft = a11 + a22, tft = a11 * a22 - a12 * a21;
+    T a11 = *A.at(hi - 1, hi - 1), a22 = *A.at(hi, hi), w = *A.at(hi - 1, hi) * *A.at(hi, hi - 1);
     if (exceptional) {
-        const T ww = fabs(a21) + fabs(*A.at(hi - 1, hi - 2));
-        sft = (T)1.5 * ww;
-        tft = ww * ww;
+        const T ww = fabs(*A.at(hi, hi - 1)) + fabs(*A.at(hi - 1, hi - 2));
+        a11 = a22 = a22 + (T)0.75 * ww;
+        w = (T)-0.4375 * ww * ww;
     }
     const T h00 = *A.at(lo, lo), h01 = *A.at(lo, lo + 1), h10 = *A.at(lo + 1, lo), h11 = *A.at(lo + 1, lo + 1);
-    bu.x0 = h00 * h00 + h01 * h10 - sft * h00 + tft;
-    bu.x1 = h10 * (h00 + h11 - sft);
-    bu.x2 = h10 * *A.at(lo + 2, lo + 1);
+    const T r = a22 - h00, s = a11 - h00;
+    bu.x0 = (r * s - w) / h10 + h01;
+    bu.x1 = h11 - h00 - r - s;
+    bu.x2 = *A.at(lo + 2, lo + 1);
     bu.b = (T)0;
 }
 
@@ -792,7 +790,7 @@ __device__ __noinline__ void hqr_global(T* Ag, const int n, double* wr, double* 
 
 template <typename T>
 __device__ void eigen_screen(T* A, const int n, T* cs, T* rs, T* v, T* part, double* wr, double* wi, DShared& sh) {
-    balance<T>(A, n, cs, rs, sh);
+    balance<T>(A, n, cs, rs, v, sh);             // (the factors are not needed: eigenvalues only)
     hessenberg<T>(A, n, v, cs, rs, part, sh);
     hqr_global<T>(A, n, wr, wi, sh);
 }
@@ -1159,8 +1157,8 @@ dyn_kernel(DevNet net, EvalArgs a, OpfOut o, double damping_min, double* scratch
             for (int w = tid; w < n * n; w += nthr) A32[w] = (float)A[w];
             if (tid == 0) dst[0] = __int_as_float(n);
             __syncthreads();
-            balance<float>(A32, n, reinterpret_cast<float*>(cs_d), reinterpret_cast<float*>(rs_d), sh,
-                           dst + ab_d_off(5 * ng - 1));
+            balance<float>(A32, n, reinterpret_cast<float*>(cs_d), reinterpret_cast<float*>(rs_d),
+                           dst + ab_d_off(5 * ng - 1), sh);
             __syncthreads();
             continue;
         }
@@ -1168,7 +1166,8 @@ dyn_kernel(DevNet net, EvalArgs a, OpfOut o, double damping_min, double* scratch
             float* A32 = reinterpret_cast<float*>(W + L.A32);
             for (int w = tid; w < n * n; w += nthr) A32[w] = (float)A[w];
             __syncthreads();
-            balance<float>(A32, n, reinterpret_cast<float*>(cs_d), reinterpret_cast<float*>(rs_d), sh);
+            balance<float>(A32, n, reinterpret_cast<float*>(cs_d), reinterpret_cast<float*>(rs_d),
+                           reinterpret_cast<float*>(v_d), sh);
             __syncthreads();
             float* slot = hbuf + (size_t)s * hstride;
             const int nmax = 5 * ng - 1;
@@ -1252,9 +1251,22 @@ __global__ void record_kernel(int nbr, int nE, EvalArgs a) {
 // update; two cluster barriers per column.  Exchange buffers alternate with the
 // column parity, so a CTA that runs ahead never overwrites what its peer still
 // reads.  The packed Hessenberg matrix goes to hbuf for hqr_smem_kernel.
-constexpr int kHsThreads = 256;
+//
+// The reflector and w = beta v^T A are indexed by absolute rows and columns, zero up to the column
+// being reduced, so a row's two updates need no masks: a lane takes two adjacent columns of each
+// group of 64, and groups left of the column are skipped.  (With a lane per column counted from
+// the reduced one, and twelve masked columns per lane whatever was left, most of the
+// instructions were masks.  118 buses, one scenario 1.69 -> 1.24 ms, 417 of them 10.1 -> 7.4 ms.)
+constexpr int kHsThreads = 512;
 constexpr int kHsWarps = kHsThreads / 32;
-constexpr int kHsCols = 12;         // columns per lane in the row pass: orders up to 32 * 12 + 1
+constexpr int kHsCols = 12;         // columns per lane in the row pass: orders up to 32 * 12
+constexpr int kHsGroups = kHsCols / 2;
+
+// row stride in shared memory: even (pairs of columns), not a multiple of 32 banks
+__host__ __device__ inline int hs_ld(int n) {
+    const int ld = (n + 1) & ~1;
+    return (ld & 31) == 0 ? ld + 2 : ld;
+}
 
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kHsThreads, 1)
 hess_cluster_kernel(EvalArgs a, OpfOut o, float* __restrict__ abuf, size_t astride, float* __restrict__ hbuf,
@@ -1263,12 +1275,13 @@ hess_cluster_kernel(EvalArgs a, OpfOut o, float* __restrict__ abuf, size_t astri
     cg::cluster_group cl = cg::this_cluster();
     const int rank = (int)cl.block_rank();
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    extern __shared__ float csm[];
-    const int hmax = (nmax + 1) / 2;
-    float* As = csm;                                  // own rows, row stride n
-    float* vb = As + (size_t)hmax * nmax;             // [2 parity][nmax] raw column k (vb[.][0] = x0)
-    float* wb = vb + 2 * nmax;                        // [2 parity][2 rank][nmax] partial v^T A
-    float* np = wb + 4 * nmax;                        // [2 parity][2 rank] partial squared norms
+    extern __shared__ __align__(16) float csm[];
+    const int hmax = (nmax + 1) / 2, ldm = hs_ld(nmax);
+    float* As = csm;                                  // own rows, row stride ld
+    float* vb = As + (size_t)hmax * ldm;              // [2 parity][ldm] reflector, by absolute row
+    float* wb = vb + 2 * ldm;                         // [2 parity][2 rank][ldm] partial v^T A, by absolute column
+    float* ws = wb + 4 * ldm;                         // [kHsSlices][ldm] this CTA's partial sums by row slices
+    float* np = ws + kHsSlices * ldm;                 // [2 parity][2 rank] partial squared norms
     __shared__ float red[kHsWarps];
     __shared__ int scen;
     float* peer_vb = cl.map_shared_rank(vb, rank ^ 1);
@@ -1288,7 +1301,7 @@ hess_cluster_kernel(EvalArgs a, OpfOut o, float* __restrict__ abuf, size_t astri
         if (s >= a.n) break;
         if (o.status[s] != 1) continue;
         float* src = abuf + (size_t)s * astride;
-        const int n = __float_as_int(src[0]);
+        const int n = __float_as_int(src[0]), ld = hs_ld(n);
         const float* Ag = src + kHqHead;
         // Householder vectors and factors for the refinement kernel: rank 0 writes them
         // over the slot's matrix, after both CTAs have loaded their rows (the first
@@ -1296,20 +1309,24 @@ hess_cluster_kernel(EvalArgs a, OpfOut o, float* __restrict__ abuf, size_t astri
         float* refl = src + kHqHead;
         float* betas = src + ab_beta_off(nmax);
         const int h = (n + 1) / 2, r0 = rank * h, r1 = min(n, r0 + h), nr = max(0, r1 - r0);
-        for (int w = tid; w < nr * n; w += kHsThreads) As[w] = Ag[(size_t)r0 * n + w];
-        __syncthreads();
+        for (int i = warp; i < nr; i += kHsWarps)
+            for (int j = lane; j < ld; j += 32) As[(size_t)i * ld + j] = (j < n) ? Ag[(size_t)(r0 + i) * n + j] : 0.0f;
+        for (int w = tid; w < 2 * ldm; w += kHsThreads) vb[w] = 0.0f;
+        // the peer writes its part of the reflector into vb: not before it is cleared
+        cl.sync();
         for (int k = 0; k + 2 < n; ++k) {
             const int par = k & 1;
-            float* v = vb + par * nmax;
-            float* pv = peer_vb + par * nmax;
+            float* v = vb + par * ldm;
+            float* pv = peer_vb + par * ldm;
             const int i0 = max(r0, k + 1);
             float t = 0.0f;
             for (int i = i0 + tid; i < r1; i += kHsThreads) {
-                const float q = As[(i - r0) * n + k];
-                v[i - k - 1] = q;
-                pv[i - k - 1] = q;
+                const float q = As[(size_t)(i - r0) * ld + k];
+                v[i] = q;
+                pv[i] = q;
                 if (i >= k + 2) t += q * q;
             }
+            if (tid < 2 && k - tid >= 0) v[k - tid] = 0.0f;   // left from two columns ago
             for (int off = 16; off; off >>= 1) t += __shfl_xor_sync(0xffffffffu, t, off);
             if (lane == 0) red[warp] = t;
             __syncthreads();
@@ -1325,7 +1342,7 @@ hess_cluster_kernel(EvalArgs a, OpfOut o, float* __restrict__ abuf, size_t astri
                 if (rank == 0 && tid == 0) betas[k] = 0.0f;
                 continue;
             }
-            const float x0 = v[0];
+            const float x0 = v[k + 1];
             const float nrm = sqrtf(x0 * x0 + tail);
             const float alpha = (x0 >= 0.0f) ? -nrm : nrm;
             const float v0 = x0 - alpha;
@@ -1333,57 +1350,98 @@ hess_cluster_kernel(EvalArgs a, OpfOut o, float* __restrict__ abuf, size_t astri
             // this CTA's copy of the reflector takes v0 in place of x0 (the peer writes only the
             // other parity's copy during this column)
             __syncthreads();
-            if (tid == 0) v[0] = v0;
+            if (tid == 0) v[k + 1] = v0;
             __syncthreads();
             if (rank == 0) {
                 float* rk = refl + refl_off(n, k);
-                for (int i = tid; i < n - k - 1; i += kHsThreads) rk[i] = v[i];
+                for (int i = tid; i < n - k - 1; i += kHsThreads) rk[i] = v[k + 1 + i];
                 if (tid == 0) betas[k] = beta;
             }
-            float* w_own = wb + (par * 2 + rank) * nmax;
-            float* w_peer = peer_wb + (par * 2 + rank) * nmax;
-            for (int j = k + 1 + tid; j < n; j += kHsThreads) {   // partial v^T A over own rows
-                float acc = 0.0f;
-                const float* col = As + (i0 - r0) * n + j;
-                const float* vv = v + (i0 - k - 1);
-                for (int i = 0; i < r1 - i0; ++i) acc += vv[i] * col[i * n];
-                w_own[j] = acc;
-                w_peer[j] = acc;
+            // partial v^T A over own rows: pairs of columns, the rows in kHsSlices slices
+            const int p0 = (k + 1) >> 1, np2 = (ld >> 1) - p0;
+            for (int w = tid; w < kHsSlices * np2; w += kHsThreads) {
+                const int sl = w / np2, j = 2 * (p0 + w - sl * np2);
+                const int m0 = i0 + (r1 - i0) * sl / kHsSlices, m1 = i0 + (r1 - i0) * (sl + 1) / kHsSlices;
+                float ax = 0.0f, ay = 0.0f, bx = 0.0f, by = 0.0f;
+                const float* col = As + (size_t)(m0 - r0) * ld + j;
+                int i = m0;
+                for (; i + 2 <= m1; i += 2, col += 2 * ld) {
+                    const float2 q = *reinterpret_cast<const float2*>(col), u = *reinterpret_cast<const float2*>(col + ld);
+                    const float v1 = v[i], v2 = v[i + 1];
+                    ax += v1 * q.x; ay += v1 * q.y;
+                    bx += v2 * u.x; by += v2 * u.y;
+                }
+                if (i < m1) {
+                    const float2 q = *reinterpret_cast<const float2*>(col);
+                    ax += v[i] * q.x; ay += v[i] * q.y;
+                }
+                *reinterpret_cast<float2*>(ws + sl * ldm + j) = make_float2(ax + bx, ay + by);
+            }
+            __syncthreads();
+            float* w_own = wb + (par * 2 + rank) * ldm;
+            float* w_peer = peer_wb + (par * 2 + rank) * ldm;
+            for (int j = 2 * p0 + tid; j < ld; j += kHsThreads) {
+                float q = 0.0f;
+#pragma unroll
+                for (int sl = 0; sl < kHsSlices; ++sl) q += ws[sl * ldm + j];
+                if (j == k) q = 0.0f;                 // the reduced column is written below
+                w_own[j] = q;
+                w_peer[j] = q;
             }
             cl.sync();                                // partial sums exchanged
-            // One pass per own row, a warp per row: the left update (rows k+1..),
-            // column k, then the right update, with the row held in registers.  Each
-            // lane keeps w and v for its columns k+1+lane+32t in registers.
-            const float* w0 = wb + (par * 2) * nmax;
-            const float* w1 = wb + (par * 2 + 1) * nmax;
-            const int mm = n - k - 1;
-            float wr_[kHsCols], vr_[kHsCols];
+            // One pass per own row, a warp per two rows: the left update (rows k+1..), the right
+            // update, then column k; a lane keeps w and v of its columns in registers.
+            const float* w0 = wb + (par * 2) * ldm;
+            const int g0 = (k + 1) >> 6, g1 = (ld + 63) >> 6;
+            float2 wv[kHsGroups], vv[kHsGroups];
 #pragma unroll
-            for (int t = 0; t < kHsCols; ++t) {
-                const int jj = lane + 32 * t;             // offset from column k+1
-                wr_[t] = (jj < mm) ? beta * (w0[k + 1 + jj] + w1[k + 1 + jj]) : 0.0f;
-                vr_[t] = (jj < mm) ? v[jj] : 0.0f;
+            for (int g = 0; g < kHsGroups; ++g) {
+                const int j = 64 * g + 2 * lane;
+                wv[g] = vv[g] = make_float2(0.0f, 0.0f);
+                if (g >= g0 && g < g1 && j >= 2 * p0 && j < ld) {
+                    const float2 q = *reinterpret_cast<const float2*>(w0 + j), u = *reinterpret_cast<const float2*>(w0 + ldm + j);
+                    wv[g] = make_float2(beta * (q.x + u.x), beta * (q.y + u.y));
+                    vv[g] = *reinterpret_cast<const float2*>(v + j);
+                }
             }
-            for (int i = warp; i < nr; i += kHsWarps) {
-                float* row = As + i * n + k + 1;
-                const int gi = r0 + i;
-                const float vi = (gi >= k + 1) ? v[gi - k - 1] : 0.0f;
-                float x[kHsCols];
-                float acc = 0.0f;
+            for (int i = 2 * warp; i < nr; i += 2 * kHsWarps) {
+                const bool two = i + 1 < nr;
+                float* row[2] = {As + (size_t)i * ld + 2 * lane, As + (size_t)(two ? i + 1 : i) * ld + 2 * lane};
+                const float vi[2] = {v[r0 + i], two ? v[r0 + i + 1] : 0.0f};
+                float2 x[2][kHsGroups];
+                float acc[2] = {0.0f, 0.0f};
 #pragma unroll
-                for (int t = 0; t < kHsCols; ++t) {
-                    const int jj = lane + 32 * t;
-                    x[t] = (jj < mm) ? row[jj] - vi * wr_[t] : 0.0f;
-                    acc += x[t] * vr_[t];
-                }
-                for (int off = 16; off; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
-                acc *= beta;
+                for (int g = 0; g < kHsGroups; ++g) {
+                    if (g < g0 || g >= g1) continue;
 #pragma unroll
-                for (int t = 0; t < kHsCols; ++t) {
-                    const int jj = lane + 32 * t;
-                    if (jj < mm) row[jj] = x[t] - acc * vr_[t];
+                    for (int q = 0; q < 2; ++q) {
+                        float2 y = make_float2(0.0f, 0.0f);
+                        if (64 * g + 2 * lane < ld) y = *reinterpret_cast<const float2*>(row[q] + 64 * g);
+                        y.x -= vi[q] * wv[g].x;
+                        y.y -= vi[q] * wv[g].y;
+                        acc[q] += y.x * vv[g].x + y.y * vv[g].y;
+                        x[q][g] = y;
+                    }
                 }
-                if (lane == 0 && gi >= k + 1) row[-1] = (gi == k + 1) ? alpha : 0.0f;
+                for (int off = 16; off; off >>= 1) {
+                    acc[0] += __shfl_xor_sync(0xffffffffu, acc[0], off);
+                    acc[1] += __shfl_xor_sync(0xffffffffu, acc[1], off);
+                }
+                acc[0] *= beta;
+                acc[1] *= beta;
+#pragma unroll
+                for (int g = 0; g < kHsGroups; ++g) {
+                    if (g < g0 || g >= g1) continue;
+#pragma unroll
+                    for (int q = 0; q < 2; ++q) {
+                        if (64 * g + 2 * lane < ld && (q == 0 || two))
+                            *reinterpret_cast<float2*>(row[q] + 64 * g) =
+                                make_float2(x[q][g].x - acc[q] * vv[g].x, x[q][g].y - acc[q] * vv[g].y);
+                    }
+                }
+                __syncwarp();
+                if (lane < (two ? 2 : 1) && r0 + i + lane > k)
+                    As[(size_t)(i + lane) * ld + k] = (r0 + i + lane == k + 1) ? alpha : 0.0f;
             }
             __syncthreads();
         }
@@ -1392,9 +1450,9 @@ hess_cluster_kernel(EvalArgs a, OpfOut o, float* __restrict__ abuf, size_t astri
         for (int i = r0 + warp; i < r1; i += kHsWarps) {
             const int j0 = hq_start(i);
             float* drow = dst + kHqHead + hq_off(n, i) - j0;
-            for (int j = j0 + lane; j < n; j += 32) drow[j] = As[(i - r0) * n + j];
+            for (int j = j0 + lane; j < n; j += 32) drow[j] = As[(size_t)(i - r0) * ld + j];
         }
-        __syncthreads();
+        cl.sync();                                    // the peer has read this CTA's exchange buffers
     }
 }
 
@@ -1417,8 +1475,6 @@ constexpr int kQrThreads = CS_QR_THREADS;
 // only need to be within kEigDelta of the exact ones (the decisive ones are refined in
 // FP64), which that normwise perturbation respects.
 constexpr int kStallIts = 40;
-// the column phase of a bulge step covers at most 2 kQrThreads rows (orders up to 32 kHsCols + 1)
-static_assert(2 * kQrThreads > 32 * kHsCols + 1, "QR column phase: at most two rows per thread");
 
 __device__ __forceinline__ void eig2f(float p, float q, float r, float s, float* re, float* im) {
     const float hm = 0.5f * (p - s);
@@ -1968,14 +2024,14 @@ static size_t refine_smem_bytes(int nmax) {
 }
 
 static size_t hess_smem_bytes(int nmax) {
-    return sizeof(float) * ((size_t)((nmax + 1) / 2) * nmax + 6 * (size_t)nmax + 4);
+    return sizeof(float) * ((size_t)((nmax + 1) / 2 + 6 + kHsSlices) * hs_ld(nmax) + 4);
 }
 
 bool dyn_split_fits(const DevNet& net, int device) {
     int optin = 0;
     if (cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, device) != cudaSuccess) return false;
     const int nmax = 5 * net.ng - 1;
-    if (nmax - 1 > 32 * kHsCols) return false;
+    if (nmax > 32 * kHsCols) return false;
     return qr_smem_bytes(nmax) + 1024 <= (size_t)optin && hess_smem_bytes(nmax) + 1024 <= (size_t)optin &&
            refine_smem_bytes(nmax) + sizeof(RfShared) + 1024 <= (size_t)optin;
 }
@@ -1994,7 +2050,9 @@ static cudaError_t launch_mode(const DevNet& net, const EvalArgs& a, OpfOut o, d
     // four per SM, fill one another's chains.  Results do not depend on the number of threads.
     // 118 buses, FP64 screen: 2,000 pairs 572 ms with four blocks of 128 threads per SM, 713 with two of 256
     // (510 now, with the one-pass Hessenberg reduction); 240 single outages 144 and 124 (114 now).
-    const int threads = grid > 2 * sms ? 128 : grid > sms ? 256 : 512;
+    // The front kernels have no such chain and move more memory per block: two blocks of 256.
+    const bool front = kMode == DYN_FRONT || kMode == DYN_FRONT_LARGE;
+    const int threads = grid <= sms ? 512 : (front || grid <= 2 * sms) ? 256 : 128;
     dyn_kernel<kMode><<<grid, threads, smem, s>>>(net, a, o, damping_min, scratch, per_cta, L, hbuf, hstride, a64,
                                                   dyn_a64_stride(net), counter);
     return cudaGetLastError();
