@@ -418,8 +418,8 @@ constexpr int kQrNB = sizeof(T) == 8 ? 8 : 12;   // measured: FP32 8 / 12 / 16, 
 constexpr int kQrCols = 32;                      // columns of a window kept in the chasing warp
 
 template <typename T>
-struct alignas(16) QrStep {                      // reflector of one step
-    T v1, v2, tau;
+struct alignas(16) QrStep {                      // reflector of one step; t1 = tau v1, t2 = tau v2
+    T v1, v2, tau, t1, t2;
 };
 template <typename T>
 struct QrSpace {                                 // in shared memory
@@ -538,10 +538,10 @@ __device__ __forceinline__ void qr_apply(T (&y)[kQrNB<T> + 2], const QrSpace<T>&
     for (int t = 0; t < kQrNB<T>; ++t) {
         if (!kFull && (t >= cnt || t < first)) continue;
         const QrStep<T> st = sp.st[t];
-        const T d = st.tau * (y[t] + st.v1 * y[t + 1] + st.v2 * y[t + 2]);
-        y[t] -= d;
-        y[t + 1] -= st.v1 * d;
-        y[t + 2] -= st.v2 * d;
+        const T d = y[t] + st.v1 * y[t + 1] + st.v2 * y[t + 2];
+        y[t] -= st.tau * d;
+        y[t + 1] -= st.t1 * d;
+        y[t + 2] -= st.t2 * d;
     }
 }
 
@@ -585,7 +585,7 @@ __device__ __forceinline__ void qr_chase(const M& A, int lo, int hi, int kw, int
         }
         const QrRefl<T> h = qr_reflector(x0, x1, x2);
         const T v1 = h.v1, v2 = h.v2, tau = h.tau, t1 = tau * v1, t2 = tau * v2;
-        sp.st[t] = {v1, v2, tau};                         // the same from every lane
+        sp.st[t] = {v1, v2, tau, t1, t2};                         // the same from every lane
         if (lane == t) sub = h.alpha;
         T da, db, dc;
         if (kCopies) {
@@ -637,51 +637,43 @@ __device__ __forceinline__ void qr_chase(const M& A, int lo, int hi, int kw, int
     if (kw + cnt == hi && lane == 0) *A.at(hi, hi - 1) = x0;
 }
 
-// The window's reflectors on the rows above it, the columns right of it, and its own rows (each from
-// its own step on).  A warp takes 32 rows or 32 columns at a time.
+// The window's reflectors on the rows above it, its own rows (each from its own step on) and the
+// columns right of it.  A warp takes 32 rows or 32 columns at a time.
 template <typename T, typename M>
 __device__ __forceinline__ void qr_strips(const M& A, int lo, int hi, int kw, int cnt, const QrSpace<T>& sp, int warp,
                                           int nwarps) {
-    const int lane = threadIdx.x & 31, nrow = kw - lo, jc = kw + kQrCols, ncol = max(0, hi + 1 - jc);
+    constexpr int NB = kQrNB<T>;
+    const int lane = threadIdx.x & 31, nrow = kw + cnt - lo, jc = kw + kQrCols, ncol = max(0, hi + 1 - jc);
     const int trow = (nrow + 31) >> 5, tcol = (ncol + 31) >> 5;
-    const bool full = cnt == kQrNB<T> && kw + kQrNB<T> + 1 <= hi;
-    for (int task = warp; task < trow + tcol + 1; task += nwarps) {
-        T y[kQrNB<T> + 2];
+    const bool full = cnt == NB && kw + NB + 1 <= hi;
+    for (int task = warp; task < trow + tcol; task += nwarps) {
+        T y[NB + 2];
         if (task < trow) {
-            const int i = lo + 32 * task + lane;
-            if (i >= kw) continue;
+            const int i = lo + 32 * task + lane, first = max(0, i - kw);
+            if (i >= kw + cnt) continue;
             T* row = A.at(i, kw);
-            if (full) {
+            if (full && lo + 32 * task + 31 < kw) {
 #pragma unroll
-                for (int c = 0; c < kQrNB<T> + 2; ++c) y[c] = row[c];
-                qr_apply<true>(y, sp, 0, kQrNB<T>);
+                for (int c = 0; c < NB + 2; ++c) y[c] = row[c];
+                qr_apply<true>(y, sp, 0, NB);
 #pragma unroll
-                for (int c = 0; c < kQrNB<T> + 2; ++c) row[c] = y[c];
+                for (int c = 0; c < NB + 2; ++c) row[c] = y[c];
             } else {
 #pragma unroll
-                for (int c = 0; c < kQrNB<T> + 2; ++c) y[c] = (c <= cnt + 1 && kw + c <= hi) ? row[c] : (T)0;
-                qr_apply<false>(y, sp, 0, cnt);
+                for (int c = 0; c < NB + 2; ++c) y[c] = (c >= first && c <= cnt + 1 && kw + c <= hi) ? row[c] : (T)0;
+                qr_apply<false>(y, sp, first, cnt);
 #pragma unroll
-                for (int c = 0; c < kQrNB<T> + 2; ++c)
-                    if (c <= cnt + 1 && kw + c <= hi) row[c] = y[c];
+                for (int c = 0; c < NB + 2; ++c)
+                    if (c >= first && c <= cnt + 1 && kw + c <= hi) row[c] = y[c];
             }
-        } else if (task < trow + tcol) {                         // (columns right of a window: it is full)
+        } else {                                                 // (columns right of a window: it is full)
             const int j = jc + 32 * (task - trow) + lane;
             if (j > hi) continue;
 #pragma unroll
-            for (int r = 0; r < kQrNB<T> + 2; ++r) y[r] = *A.at(kw + r, j);
-            qr_apply<true>(y, sp, 0, kQrNB<T>);
+            for (int r = 0; r < NB + 2; ++r) y[r] = *A.at(kw + r, j);
+            qr_apply<true>(y, sp, 0, NB);
 #pragma unroll
-            for (int r = 0; r < kQrNB<T> + 2; ++r) *A.at(kw + r, j) = y[r];
-        } else {
-            if (lane >= cnt) continue;
-            T* row = A.at(kw + lane, kw);
-#pragma unroll
-            for (int c = 0; c < kQrNB<T> + 2; ++c) y[c] = (c >= lane && c <= cnt + 1 && kw + c <= hi) ? row[c] : (T)0;
-            qr_apply<false>(y, sp, lane, cnt);
-#pragma unroll
-            for (int c = 0; c < kQrNB<T> + 2; ++c)
-                if (c >= lane && c <= cnt + 1 && kw + c <= hi) row[c] = y[c];
+            for (int r = 0; r < NB + 2; ++r) *A.at(kw + r, j) = y[r];
         }
     }
 }
@@ -708,12 +700,12 @@ __device__ __forceinline__ void qr_start(const M& A, int lo, int hi, bool except
     bu.b = (T)0;
 }
 
-// Whole sweep by the block: the warp `chaser` starts and chases, all threads take the strips.
+// Whole sweep by the block: warp 0 starts and chases, all threads take the strips.  (Chasing with a
+// different warp in each of the blocks that share an SM measured the same.)
 template <typename T, typename M>
-__device__ __forceinline__ void qr_sweep(const M& A, int lo, int hi, bool exceptional, QrSpace<T>& sp, int nthreads,
-                                         int chaser) {
-    const int tid = threadIdx.x, nthr = blockDim.x;
-    const bool mine = (tid >> 5) == chaser;
+__device__ __forceinline__ void qr_sweep(const M& A, int lo, int hi, bool exceptional, QrSpace<T>& sp, int nthreads) {
+    const int tid = threadIdx.x;
+    const bool mine = tid < 32;
     QrBulge<T> bu{};
     if (mine) qr_start<T>(A, lo, hi, exceptional, bu);
     for (int kw = lo; kw < hi; kw += kQrNB<T>) {
@@ -736,10 +728,6 @@ __device__ __noinline__ void hqr_global(T* Ag, const int n, double* wr, double* 
     __shared__ QrSpace<T> sp;
     const int tid = threadIdx.x, nthr = blockDim.x;
     const DenseMat<T> A{Ag, n};
-    // The blocks resident on an SM chase with different warps: an FP64 chase fills its sub-partition's
-    // FP64 pipe, and warp w of a block sits on sub-partition w mod 4 (consecutive blocks, or blocks one
-    // grid round apart, share an SM).
-    const int chaser = (blockIdx.x + blockIdx.x / 152) & 3;
     const T eps = (sizeof(T) == 8) ? (T)kEps : (T)kDeflTol;              // deflation tolerance
     double hmax;
     {
@@ -783,7 +771,7 @@ __device__ __noinline__ void hqr_global(T* Ag, const int n, double* wr, double* 
             break;
         }
         ++its;
-        qr_sweep<T>(A, lo, hi, its == 10 || its == 20, sp, nthr, chaser);
+        qr_sweep<T>(A, lo, hi, its == 10 || its == 20, sp, nthr);
     }
     __syncthreads();                               // eigenvalues and sh.fail written by thread 0
 }
@@ -1587,7 +1575,7 @@ hqr_smem_kernel(EvalArgs a, OpfOut o, const float* __restrict__ hbuf, size_t hst
             }
             ++its;
             __syncthreads();              // every warp has read the block before the sweep writes
-            qr_sweep<float>(A, lo, hi, its % 10 == 0, sp, kQrThreads, 0);  // exceptional shift every tenth sweep
+            qr_sweep<float>(A, lo, hi, its % 10 == 0, sp, kQrThreads);  // exceptional shift every tenth sweep
         }
         __syncthreads();                                   // wr, wi written by thread 0
         // statistics over all eigenvalues: max Re, min damping ratio
