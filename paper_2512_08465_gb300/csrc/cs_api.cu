@@ -40,6 +40,7 @@ int64_t default_chunk(const cs_ctx* ctx, const Network& net) {
 }
 
 namespace {
+constexpr size_t kDynScratch = (size_t)2 << 30;      // bytes, see grids()
 constexpr int kCounters = 6;      // work counters of one chunk: OPF, then five small-signal kernels
 struct Grids {
     int g_opf, g_dyn;
@@ -63,6 +64,15 @@ Grids grids(const cs_ctx* ctx, const Network& net, int64_t cn) {
     g.g_dyn = (int)std::max<int64_t>(1, std::min<int64_t>((int64_t)ctx->sms * cap_dyn, cn));
     g.per_opf = opf_scratch_doubles(dn);
     g.per_dyn = dyn_scratch_doubles(dn);
+    if (ctx->opt.ctas_per_sm <= 0 && net.dyn_cap <= 0) {
+        // The OPF scratch (or two small-signal CTAs per SM) sets the workspace.  The default of four
+        // may exceed it up to kDynScratch, unless the device memory is budgeted: on 300 buses the four
+        // need 1.35 GB for the two's 0.74 GB, on 1,000 buses 14.7 GB for 7.4 GB (two there).
+        const size_t two = g.per_dyn * (size_t)std::min<int64_t>((int64_t)ctx->sms * 2, cn);
+        size_t lim = std::max(g.per_opf * g.g_opf, two);
+        if (ctx->opt.hbm_budget <= 0) lim = std::max(lim, kDynScratch / sizeof(double));
+        g.g_dyn = (int)std::min<size_t>(g.g_dyn, std::max<size_t>(1, lim / std::max<size_t>(1, g.per_dyn)));
+    }
     return g;
 }
 bool split_path(const cs_ctx* ctx, const DevNet& dn) {
@@ -443,7 +453,9 @@ cs_status autotune_network(cs_ctx* ctx, Network* net) {
         }
         ctx->ev_used = 0;
         if (t < 0) continue;
-        if (ms[1] < best_opf) { best_opf = ms[1]; pick_opf = net->opf_cap; }
+        // (a shape whose smaller neighbour holds the whole sample launches the same grid: no candidate)
+        const bool same = net->opf_cap > 1 && (int64_t)(net->opf_cap - 1) * ctx->sms >= ns;
+        if (!same && ms[1] < best_opf) { best_opf = ms[1]; pick_opf = net->opf_cap; }
         if (ms[2] < best_dyn) { best_dyn = ms[2]; pick_dyn = net->dyn_cap; }
     }
     net->opf_cap = pick_opf;

@@ -26,8 +26,9 @@
 //     5x5 block of A;
 //  4. balancing by powers of two, Householder Hessenberg reduction, Francis
 //     double-shift QR (eigenvalues only), with the same steps and thresholds
-//     as the textbook algorithm; A lives in the CTA's global scratch (the
-//     resident CTAs' matrices together fit in the 129 MB L2);
+//     as the textbook algorithm, the Hessenberg reduction in one pass over A
+//     per column and the QR sweeps in windows of several steps; A lives in
+//     the CTA's global scratch;
 //  5. max Re and min damping ratio over all eigenvalues, classify.
 // Angle reference: every rotor angle is referred to the first in-service
 // machine (delta'_k = delta_k - delta_0, d delta'_k/dt = ws (omega_k - omega_0),
@@ -87,7 +88,9 @@ DLay make_dlayout(const DevNet& n) {
     L.A32 = take((25L * n.ng * n.ng + 1) / 2);
     o = (o + 31) & ~31;
     L.wr = take(5L * n.ng); L.wi = take(5L * n.ng); L.v = take(5L * n.ng);
-    L.hp = take(8L * 5 * n.ng);
+    // partial sums of the Hessenberg slices: on the reduction's right-hand sides, which nothing reads once
+    // the state matrix is formed, where they fit
+    L.hp = 2L * n.nb >= 40 ? L.rhs : take(8L * 5 * n.ng);
     L.total = (o + 31) & ~31;
     return L;
 }
@@ -408,7 +411,8 @@ __device__ __noinline__ void hessenberg(T* A, const int n, T* v, T* w, T* vn, T*
 //    reflectors) and per column to the right (left reflectors), with the row's or column's kQrNB + 2
 //    entries in registers.
 // So a window costs two barriers where a step cost two, and an entry is loaded and stored once per
-// window.  What bounds it is the chase, a chain of dependent instructions of one warp (FP32 ~350
+// window.  A reflector is kept with tau v1 and tau v2, so a row or a column takes five multiply-adds
+// of it (seven operations before: 2,000 pairs in FP64 591 -> 576 ms).  What bounds it is the chase, a chain of dependent instructions of one warp (FP32 ~350
 // cycles a step, FP64 ~2,900; the strips take 100 and 1,000).  118 buses: FP32 QR of one scenario
 // from shared memory 8.2 -> 5.4 ms.
 //
@@ -1446,9 +1450,9 @@ hess_cluster_kernel(EvalArgs a, OpfOut o, float* __restrict__ abuf, size_t astri
 
 // ---------------------------------------------------------------------------
 // FP32 screen, last part: Francis double-shift QR of the packed Hessenberg
-// matrix held in shared memory (one scenario per CTA, one CTA per SM).  Every
-// thread carries the same loop state (lo, hi, shifts, reflector), computed
-// redundantly from shared memory in FP32, so a bulge step costs two barriers.
+// matrix held in shared memory (one scenario per CTA, one CTA per SM), the
+// sweeps in windows (qr_sweep).  Every thread carries the same loop state
+// (lo, hi, sweep count), computed redundantly from shared memory.
 // Exceptional shifts come every tenth sweep without a deflation, and a stalled
 // window also deflates at the normwise FP32 level (kStallIts).  A scenario whose
 // QR does not converge is marked for the FP64 re-run; the others get their
@@ -2037,7 +2041,7 @@ static cudaError_t launch_mode(const DevNet& net, const EvalArgs& a, OpfOut o, d
     // few scenarios a block of many threads shortens the wide phases, with many scenarios small blocks,
     // four per SM, fill one another's chains.  Results do not depend on the number of threads.
     // 118 buses, FP64 screen: 2,000 pairs 572 ms with four blocks of 128 threads per SM, 713 with two of 256
-    // (510 now, with the one-pass Hessenberg reduction); 240 single outages 144 and 124 (114 now).
+    // (485 now, with the one-pass Hessenberg reduction); 240 single outages 144 and 124 (112 now).
     // The front kernels have no such chain and move more memory per block: two blocks of 256.
     const bool front = kMode == DYN_FRONT || kMode == DYN_FRONT_LARGE;
     const int threads = grid <= sms ? 512 : (front || grid <= 2 * sms) ? 256 : 128;

@@ -28,9 +28,10 @@
 //    left-looking update lists, built on the host at load time), with the
 //    4x4 pivot blocks inverted by LU with partial pivoting.  Columns
 //    of one elimination-tree level are independent, so a level is one
-//    parallel step of the CTA (16 threads per target block).  The narrow
-//    upper levels leave most threads at barriers, so CTAs are small (128
-//    threads) and three are resident per SM to overlap one another's waits;
+//    parallel step of the CTA: its block updates are cut into equal shares
+//    for eight groups of 16 threads, an entry of the target per thread.  The
+//    narrow upper levels leave most threads at barriers, so CTAs are small
+//    (128 threads) and four are resident per SM to overlap one another's waits;
 //  * every branch quantity (flows, first and second derivatives of both end
 //    powers, the weighted 4x4 Hessian) is computed once per iteration by one
 //    thread from the branch's own four voltage variables and gathered by
