@@ -407,14 +407,15 @@ __device__ __noinline__ void hessenberg(T* A, const int n, T* v, T* w, T* vn, T*
 //  * chase: one warp carries the bulge through the window with the window's rows in registers, a
 //    lane per column: left reflectors act within a lane, right reflectors act as far as the next
 //    reflector needs them.
-//  * strips: all threads apply the window's kQrNB reflectors to the rest, a thread per row (right
+//  * strips: the other warps apply the window's kQrNB reflectors to the rest, a thread per row (right
 //    reflectors) and per column to the right (left reflectors), with the row's or column's kQrNB + 2
 //    entries in registers.
 // So a window costs two barriers where a step cost two, and an entry is loaded and stored once per
 // window.  A reflector is kept with tau v1 and tau v2, so a row or a column takes five multiply-adds
-// of it (seven operations before: 2,000 pairs in FP64 591 -> 576 ms).  What bounds it is the chase, a chain of dependent instructions of one warp (FP32 ~350
-// cycles a step, FP64 ~2,900; the strips take 100 and 1,000).  118 buses: FP32 QR of one scenario
-// from shared memory 8.2 -> 5.4 ms.
+// of it (seven operations before: 2,000 pairs in FP64 591 -> 576 ms).  What bounds it is the chase, a
+// chain of dependent instructions of one warp (FP32 ~350 cycles a step, FP64 ~2,900; the strips take
+// 100 and 1,000, beside it).  118 buses: FP32 QR of one scenario from shared memory 8.2 -> 5.4 ms with
+// windows, 4.3 with two sweeps at a time and the strips beside the chase (qr_sweep).
 //
 // Reflector of (x0, x1, x2): I - tau v v^T with v = (1, v1, v2), tau = 1 + |x0| / |x|.
 template <typename T>
@@ -559,8 +560,8 @@ __device__ __forceinline__ void qr_apply(T (&y)[kQrNB<T> + 2], const QrSpace<T>&
 // In FP32 the chain from one reflector to the next runs on copies of its few entries that every
 // lane keeps: rows k .. k + 2 of columns k and k + 1, and column k + 2, fetched before the reflector
 // is known.  An FP64 instruction takes longer than a shuffle, so there the entries are fetched.
-template <bool kFull, typename T, typename M>
-__device__ __forceinline__ void qr_chase(const M& A, int lo, int hi, int kw, int cnt, QrBulge<T>& bu, QrSpace<T>& sp) {
+template <typename T, typename M>
+__device__ __forceinline__ void qr_chase_full(const M& A, int lo, int hi, int kw, QrBulge<T>& bu, QrSpace<T>& sp) {
     constexpr int NB = kQrNB<T>;
     constexpr bool kCopies = sizeof(T) == 4;
     const unsigned all = 0xffffffffu;
@@ -568,7 +569,7 @@ __device__ __forceinline__ void qr_chase(const M& A, int lo, int hi, int kw, int
     T w[NB + 3];
 #pragma unroll
     for (int r = 0; r < NB + 3; ++r)
-        w[r] = ((kFull || kw + r <= hi) && col <= hi && lane + 1 >= r) ? *A.at(kw + r, col) : (T)0;
+        w[r] = (col <= hi && lane + 1 >= r) ? *A.at(kw + r, col) : (T)0;
     if (lane == 0) w[2] = bu.b;
     T x0 = bu.x0, x1 = bu.x1, x2 = bu.x2, sub = 0;        // sub: subdiagonal entry (kw + lane, kw + lane - 1)
     T m00 = 0, m01 = 0, m10 = 0, m11 = 0, m20 = 0, m21 = 0;
@@ -579,7 +580,6 @@ __device__ __forceinline__ void qr_chase(const M& A, int lo, int hi, int kw, int
     }
 #pragma unroll
     for (int t = 0; t < NB; ++t) {
-        if (!kFull && t >= cnt) break;
         T c0 = 0, c1 = 0, c2 = 0, s3 = 0;
         if (kCopies) {
             c0 = __shfl_sync(all, w[t], t + 2);
@@ -630,33 +630,145 @@ __device__ __forceinline__ void qr_chase(const M& A, int lo, int hi, int kw, int
             x2 = __shfl_sync(all, w[t + 3], t);
         }
     }
-    bu = QrBulge<T>{x0, x1, x2, kCopies ? m20 : kFull ? __shfl_sync(all, w[NB + 2], NB) : (T)0};
+    bu = QrBulge<T>{x0, x1, x2, kCopies ? m20 : __shfl_sync(all, w[NB + 2], NB)};
     // a column of the window is final on and above its diagonal; its subdiagonal entry is the next
     // step's alpha (the last one's, the next window's, or x0 at the end of the sweep)
 #pragma unroll
     for (int r = 0; r < NB + 3; ++r)
-        if ((kFull || kw + r <= hi) && col <= hi && (lane >= r || (lane + 1 == r && lane >= cnt)))
+        if (col <= hi && (lane >= r || (lane + 1 == r && lane >= NB)))
             *A.at(kw + r, col) = w[r];
+    if (lane < NB && col > lo) *A.at(col, col - 1) = sub;
+}
+
+//
+// qr_chase_full takes a window that ends three rows above the block's end or higher, unrolled; qr_chase any, in a
+// loop of kQrUnroll steps with the rows in a rolling buffer.  The size of the code counts: with all SMs at
+// it a warp waits for its instructions (118 buses, three scenarios on each SM: 15.0 ms with both kinds
+// of windows unrolled and the strips inlined four times, 13.4 like this; one scenario alone took 4.1 and
+// 4.4 ms.  Everything rolled: 15.0 and 4.9).
+constexpr int kQrUnroll = 4;
+template <typename T, typename M>
+__device__ __forceinline__ void qr_chase(const M& A, int lo, int hi, int kw, int cnt, QrBulge<T>& bu, QrSpace<T>& sp) {
+    constexpr int NB = kQrNB<T>, U = kQrUnroll;
+    static_assert(NB % U == 0 && U >= 3, "");
+    constexpr bool kCopies = sizeof(T) == 4;
+    const unsigned all = 0xffffffffu;
+    const int lane = threadIdx.x & 31, col = kw + lane;
+    auto load = [&](int r) -> T {
+        return (kw + r <= hi && col <= hi && lane + 1 >= r) ? *A.at(kw + r, col) : (T)0;
+    };
+    // a column of the window is final on and above its diagonal; its subdiagonal entry is the next
+    // step's alpha (the last one's, the next window's, or x0 at the end of the sweep)
+    auto store = [&](int r, T x) {
+        if (kw + r <= hi && col <= hi && (lane >= r || (lane + 1 == r && lane >= cnt))) *A.at(kw + r, col) = x;
+    };
+    T w[U + 3];                                           // rows t0 ..
+#pragma unroll
+    for (int r = 0; r < U + 3; ++r) w[r] = load(r);
+    if (lane == 0) w[2] = bu.b;
+    T x0 = bu.x0, x1 = bu.x1, x2 = bu.x2, sub = 0;        // sub: subdiagonal entry (kw + lane, kw + lane - 1)
+    T m00 = 0, m01 = 0, m10 = 0, m11 = 0, m20 = 0, m21 = 0;
+    if (kCopies) {
+        m00 = __shfl_sync(all, w[0], 0); m01 = __shfl_sync(all, w[0], 1);
+        m10 = __shfl_sync(all, w[1], 0); m11 = __shfl_sync(all, w[1], 1);
+        m20 = bu.b;                      m21 = __shfl_sync(all, w[2], 1);
+    }
+#pragma unroll 1
+    for (int t0 = 0; t0 < cnt; t0 += U) {
+        T next[U];                                        // rows of the steps after these
+#pragma unroll
+        for (int u = 0; u < U; ++u) next[u] = t0 + U < NB ? load(t0 + U + 3 + u) : (T)0;
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int t = t0 + u;
+            if (t >= cnt) break;
+            T c0 = 0, c1 = 0, c2 = 0, s3 = 0;
+            if (kCopies) {
+                c0 = __shfl_sync(all, w[u], t + 2);
+                c1 = __shfl_sync(all, w[u + 1], t + 2);
+                c2 = __shfl_sync(all, w[u + 2], t + 2);
+                s3 = __shfl_sync(all, w[u + 3], t + 2);
+            }
+            const QrRefl<T> h = qr_reflector(x0, x1, x2);
+            const T v1 = h.v1, v2 = h.v2, tau = h.tau, t1 = tau * v1, t2 = tau * v2;
+            sp.st[t] = {v1, v2, tau, t1, t2};             // the same from every lane
+            if (lane == t) sub = h.alpha;
+            T da, db, dc;
+            if (kCopies) {
+                const T d0 = m00 + v1 * m10 + v2 * m20, d1 = m01 + v1 * m11 + v2 * m21, d2 = c0 + v1 * c1 + v2 * c2;
+                const T n10 = m10 - t1 * d0, n20 = m20 - t2 * d0, n11 = m11 - t1 * d1, n21 = m21 - t2 * d1,
+                        n12 = c1 - t1 * d2, n22 = c2 - t2 * d2;
+                da = n10 + v1 * n11 + v2 * n12;
+                db = n20 + v1 * n21 + v2 * n22;
+                dc = v2 * s3;
+                x0 = n10 - tau * da;
+                x1 = n20 - tau * db;
+                x2 = -(tau * dc);
+                m00 = n11 - t1 * da; m01 = n12 - t2 * da;
+                m10 = n21 - t1 * db; m11 = n22 - t2 * db;
+                m20 = -(t1 * dc);    m21 = s3 - t2 * dc;
+            }
+            const T d = w[u] + v1 * w[u + 1] + v2 * w[u + 2]; // left, rows kw + t ..
+            w[u] -= tau * d;
+            w[u + 1] -= t1 * d;
+            w[u + 2] -= t2 * d;
+            if (!kCopies) {                               // right, the three rows below
+                const T a0 = __shfl_sync(all, w[u + 1], t), a1 = __shfl_sync(all, w[u + 1], t + 1),
+                        a2 = __shfl_sync(all, w[u + 1], t + 2);
+                const T b0 = __shfl_sync(all, w[u + 2], t), b1 = __shfl_sync(all, w[u + 2], t + 1),
+                        b2 = __shfl_sync(all, w[u + 2], t + 2);
+                da = a0 + v1 * a1 + v2 * a2;
+                db = b0 + v1 * b1 + v2 * b2;
+                dc = v2 * __shfl_sync(all, w[u + 3], t + 2);
+            }
+            // (column kw + t itself is the next bulge column: only needed as x)
+            const T co = lane == t + 1 ? t1 : lane == t + 2 ? t2 : kCopies ? (T)0 : lane == t ? tau : (T)0;
+            w[u + 1] -= co * da;
+            w[u + 2] -= co * db;
+            w[u + 3] -= co * dc;
+            if (!kCopies) {
+                x0 = __shfl_sync(all, w[u + 1], t);
+                x1 = __shfl_sync(all, w[u + 2], t);
+                x2 = __shfl_sync(all, w[u + 3], t);
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) store(t0 + u, w[u]);
+#pragma unroll
+        for (int r = 0; r < 3; ++r) w[r] = w[r + U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) w[u + 3] = next[u];
+    }
+    const int end = (cnt + U - 1) / U * U;
+    bu = QrBulge<T>{x0, x1, x2, kCopies ? m20 : __shfl_sync(all, w[2], NB)};   // (the last window's is not used)
+#pragma unroll
+    for (int r = 0; r < 3; ++r) store(end + r, w[r]);
     if (lane < cnt && col > lo) *A.at(col, col - 1) = sub;
     if (kw + cnt == hi && lane == 0) *A.at(hi, hi - 1) = x0;
 }
 
-// The window's reflectors on the rows above it, its own rows (each from its own step on) and the
-// columns right of it.  A warp takes 32 rows or 32 columns at a time.
+// One window's strips: its reflectors on 32 of the rows above it and its own (each from its own step
+// on), task < rows(), or on 32 of the columns right of it, task - rows() < cols().
 template <typename T, typename M>
-__device__ __forceinline__ void qr_strips(const M& A, int lo, int hi, int kw, int cnt, const QrSpace<T>& sp, int warp,
-                                          int nwarps) {
-    constexpr int NB = kQrNB<T>;
-    const int lane = threadIdx.x & 31, nrow = kw + cnt - lo, jc = kw + kQrCols, ncol = max(0, hi + 1 - jc);
-    const int trow = (nrow + 31) >> 5, tcol = (ncol + 31) >> 5;
-    const bool full = cnt == NB && kw + NB + 1 <= hi;
-    for (int task = warp; task < trow + tcol; task += nwarps) {
+struct QrStrips {
+    static constexpr int NB = kQrNB<T>;
+    const M& A;
+    const QrSpace<T>& sp;
+    int lo, hi, kw, cnt;
+    __device__ QrStrips(const M& A_, const QrSpace<T>& sp_, int lo_, int hi_, int kw_)
+        : A(A_), sp(sp_), lo(lo_), hi(hi_), kw(kw_), cnt(min(NB, hi_ - kw_)) {}
+    __device__ bool live() const { return kw >= lo && kw < hi; }
+    __device__ int rows() const { return (kw + cnt - lo + 31) >> 5; }
+    __device__ int cols() const { return (max(0, hi + 1 - kw - kQrCols) + 31) >> 5; }
+    __device__ int far() const { return live() ? rows() + max(0, cols() - 1) : 0; }   // all but the nearest columns
+    __device__ __forceinline__ void run(int task) const {
+        const int lane = threadIdx.x & 31;
         T y[NB + 2];
-        if (task < trow) {
+        if (task < rows()) {
             const int i = lo + 32 * task + lane, first = max(0, i - kw);
-            if (i >= kw + cnt) continue;
+            if (i >= kw + cnt) return;
             T* row = A.at(i, kw);
-            if (full && lo + 32 * task + 31 < kw) {
+            if (cnt == NB && kw + NB + 1 <= hi && lo + 32 * task + 31 < kw) {
 #pragma unroll
                 for (int c = 0; c < NB + 2; ++c) y[c] = row[c];
                 qr_apply<true>(y, sp, 0, NB);
@@ -671,8 +783,8 @@ __device__ __forceinline__ void qr_strips(const M& A, int lo, int hi, int kw, in
                     if (c >= first && c <= cnt + 1 && kw + c <= hi) row[c] = y[c];
             }
         } else {                                                 // (columns right of a window: it is full)
-            const int j = jc + 32 * (task - trow) + lane;
-            if (j > hi) continue;
+            const int j = kw + kQrCols + 32 * (task - rows()) + lane;
+            if (j > hi) return;
 #pragma unroll
             for (int r = 0; r < NB + 2; ++r) y[r] = *A.at(kw + r, j);
             qr_apply<true>(y, sp, 0, NB);
@@ -680,7 +792,7 @@ __device__ __forceinline__ void qr_strips(const M& A, int lo, int hi, int kw, in
             for (int r = 0; r < NB + 2; ++r) *A.at(kw + r, j) = y[r];
         }
     }
-}
+};
 
 // First column of the double-shift step, (H - a I)(H - b I) e1 / h10 of the block lo..hi, a and b the
 // eigenvalues of its trailing 2x2 block (or, if exceptional, a pair off its last entry by the size of
@@ -688,39 +800,92 @@ __device__ __forceinline__ void qr_strips(const M& A, int lo, int hi, int kw, in
 // and product, a block whose eigenvalues differ by little (the exciters' cluster near -1/T_A) loses
 // the differences to cancellation in FP32 and its sweeps go nowhere (118 buses: 331 -> 276 sweeps a
 // scenario, and the scenario in 20,000 that ran to the sweep limit converges).
+template <typename T>
+struct QrShift {
+    T a11, a22, w;                               // trailing 2x2 block: diagonal, product of the off-diagonal
+};
 template <typename T, typename M>
-__device__ __forceinline__ void qr_start(const M& A, int lo, int hi, bool exceptional, QrBulge<T>& bu) {
-    T a11 = *A.at(hi - 1, hi - 1), a22 = *A.at(hi, hi), w = *A.at(hi - 1, hi) * *A.at(hi, hi - 1);
+__device__ __forceinline__ QrShift<T> qr_shift(const M& A, int hi, bool exceptional) {
+    QrShift<T> q{*A.at(hi - 1, hi - 1), *A.at(hi, hi), *A.at(hi - 1, hi) * *A.at(hi, hi - 1)};
     if (exceptional) {
         const T ww = fabs(*A.at(hi, hi - 1)) + fabs(*A.at(hi - 1, hi - 2));
-        a11 = a22 = a22 + (T)0.75 * ww;
-        w = (T)-0.4375 * ww * ww;
+        q.a11 = q.a22 = q.a22 + (T)0.75 * ww;
+        q.w = (T)-0.4375 * ww * ww;
     }
+    return q;
+}
+template <typename T, typename M>
+__device__ __forceinline__ void qr_start(const M& A, int lo, const QrShift<T>& q, QrBulge<T>& bu) {
     const T h00 = *A.at(lo, lo), h01 = *A.at(lo, lo + 1), h10 = *A.at(lo + 1, lo), h11 = *A.at(lo + 1, lo + 1);
-    const T r = a22 - h00, s = a11 - h00;
-    bu.x0 = (r * s - w) / h10 + h01;
+    const T r = q.a22 - h00, s = q.a11 - h00;
+    bu.x0 = (r * s - q.w) / h10 + h01;
     bu.x1 = h11 - h00 - r - s;
     bu.x2 = *A.at(lo + 2, lo + 1);
     bu.b = (T)0;
 }
 
-// Whole sweep by the block: warp 0 starts and chases, all threads take the strips.  (Chasing with a
-// different warp in each of the blocks that share an SM measured the same.)
-template <typename T, typename M>
-__device__ __forceinline__ void qr_sweep(const M& A, int lo, int hi, bool exceptional, QrSpace<T>& sp, int nthreads) {
-    const int tid = threadIdx.x;
-    const bool mine = tid < 32;
+// Whole sweep by the block, or (two) two sweeps, the second one kQrLag steps behind the first with the
+// same shifts.  What bounds a sweep is the chase, a serial chain of one warp, so everything else runs
+// beside it: warp 0 (and warp 1, the second sweep) chases a window while the other warps apply the strips
+// of the window before; only the 32 columns nearest to a window, which the next one starts in, wait for
+// the chase and are waited for.
+//
+// Where the two sweeps meet: the second one's chase ends left of the columns that the first one's
+// right reflectors mix (kQrLag - kQrNB >= kQrCols), and its near columns hold all or none of them, so no
+// right reflector mixes columns with and without the second one's left reflectors.
+//
+// The shifts of the second sweep are a sweep old: 118 buses, orders 259 .. 269: 306 sweeps a matrix
+// instead of 274, in little more than half the chases.  (Eigenvalues of the trailing 4x4 block as shifts:
+// 303 sweeps, and a serial eigenvalue problem for each pair.  In FP64, whose sweeps at two or more blocks
+// per SM are bound by the pipe and not by the chase, two at a time are not used.)  From blocks of kQrPair
+// on the lag is worth it; 44, 60 and 90 measure the same.
+// 118 buses, FP32 QR of one scenario 5.4 -> 4.3 ms, 10,000 pairs mixed 883 -> 817 ms; FP64, 240 single
+// outages 133 -> 129 ms, 2,000 pairs 576 -> 565 ms.
+template <typename T>
+constexpr int kQrLag = (kQrCols + 2 * kQrNB<T> - 1) / kQrNB<T> * kQrNB<T>;
+static_assert(kQrLag<float> + kQrNB<float> + 2 <= 2 * kQrCols && kQrLag<double> + kQrNB<double> + 2 <= 2 * kQrCols,
+              "the second sweep's near columns hold the first one's window");
+constexpr int kQrPair = 60;
+template <bool kTwo, typename T, typename M>
+__device__ __forceinline__ void qr_sweep(const M& A, int lo, int hi, bool exceptional, bool two,
+                                         QrSpace<T> (&sp)[2][2], int nthreads) {
+    constexpr int NB = kQrNB<T>;
+    const int sweeps = kTwo && two ? 2 : 1;
+    const int warp = threadIdx.x >> 5, nworkers = (nthreads >> 5) - sweeps;
+    const int last = hi + (sweeps - 1) * kQrLag<T>;
     QrBulge<T> bu{};
-    if (mine) qr_start<T>(A, lo, hi, exceptional, bu);
-    for (int kw = lo; kw < hi; kw += kQrNB<T>) {
-        const int cnt = min(kQrNB<T>, hi - kw);
-        if (mine) {
-            if (kw + kQrNB<T> + 2 <= hi) qr_chase<true>(A, lo, hi, kw, cnt, bu, sp);
-            else qr_chase<false>(A, lo, hi, kw, cnt, bu, sp);
+    QrShift<T> q{};
+    if (warp < sweeps) q = qr_shift<T>(A, hi, exceptional);
+    int par = 0;
+    for (int ka = lo;; ka += NB, par ^= 1) {                      // (the last round: strips only)
+        const int kw = ka - warp * kQrLag<T>;                     // of a chasing warp
+        if (warp < sweeps && kw >= lo && kw < hi) {
+            if (kw == lo) qr_start<T>(A, lo, q, bu);
+            if (kw + NB + 2 <= hi) qr_chase_full(A, lo, hi, kw, bu, sp[warp][par]);
+            else qr_chase(A, lo, hi, kw, min(NB, hi - kw), bu, sp[warp][par]);
         }
-        __syncthreads();
-        qr_strips<T>(A, lo, hi, kw, cnt, sp, tid >> 5, nthreads >> 5);
-        __syncthreads();
+        // One loop (one copy of the strips' code) for both kinds: the windows' before, but for their nearest
+        // columns, by the other warps, then, after a barrier, the nearest of these by the chasing warps.
+#pragma unroll 1
+        for (int near = 0; near < 2; ++near) {
+            int task = 0, n = 0, na = 0;
+            if (near) {
+                n = warp < sweeps && kw >= lo && kw + kQrCols <= hi;
+            } else if (warp >= sweeps) {
+                na = n = QrStrips<T, M>(A, sp[0][0], lo, hi, ka - NB).far();
+                if (sweeps == 2) n += QrStrips<T, M>(A, sp[0][0], lo, hi, ka - NB - kQrLag<T>).far();
+                task = warp - sweeps;
+            }
+            for (; task < n; task += nworkers) {                  // (near: one)
+                const int second = !kTwo ? 0 : near ? warp : task >= na;
+                const QrStrips<T, M> st(A, sp[second][near ? par : par ^ 1], lo, hi,
+                                        near ? kw : ka - NB - second * kQrLag<T>);
+                const int t = task - second * na, rows = st.rows();
+                st.run(near ? rows : t < rows ? t : t + 1);
+            }
+            __syncthreads();
+            if (ka >= last) return;
+        }
     }
 }
 
@@ -729,7 +894,7 @@ __device__ __forceinline__ void qr_sweep(const M& A, int lo, int hi, bool except
 // sh.fail = 2 if it does not converge in 30 n sweeps.
 template <typename T>
 __device__ __noinline__ void hqr_global(T* Ag, const int n, double* wr, double* wi, DShared& sh) {
-    __shared__ QrSpace<T> sp;
+    __shared__ QrSpace<T> sp[2][2];
     const int tid = threadIdx.x, nthr = blockDim.x;
     const DenseMat<T> A{Ag, n};
     const T eps = (sizeof(T) == 8) ? (T)kEps : (T)kDeflTol;              // deflation tolerance
@@ -775,7 +940,7 @@ __device__ __noinline__ void hqr_global(T* Ag, const int n, double* wr, double* 
             break;
         }
         ++its;
-        qr_sweep<T>(A, lo, hi, its == 10 || its == 20, sp, nthr);
+        qr_sweep<false, T>(A, lo, hi, its == 10 || its == 20, false, sp, nthr);
     }
     __syncthreads();                               // eigenvalues and sh.fail written by thread 0
 }
@@ -1491,7 +1656,7 @@ hqr_smem_kernel(EvalArgs a, OpfOut o, const float* __restrict__ hbuf, size_t hst
                 double damping_min, float* __restrict__ cand, int* counter) {
     extern __shared__ float qsm[];
     __shared__ float red[2][kQrThreads / 32];
-    __shared__ QrSpace<float> sp;
+    __shared__ QrSpace<float> sp[2][2];
     __shared__ int scen;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     float* H = qsm;                                           // hq_off(nmax, nmax) floats
@@ -1579,7 +1744,8 @@ hqr_smem_kernel(EvalArgs a, OpfOut o, const float* __restrict__ hbuf, size_t hst
             }
             ++its;
             __syncthreads();              // every warp has read the block before the sweep writes
-            qr_sweep<float>(A, lo, hi, its % 10 == 0, sp, kQrThreads);  // exceptional shift every tenth sweep
+            const bool exceptional = its % 10 == 0;               // every tenth time without a deflation
+            qr_sweep<true, float>(A, lo, hi, exceptional, !exceptional && hi - lo >= kQrPair, sp, kQrThreads);
         }
         __syncthreads();                                   // wr, wi written by thread 0
         // statistics over all eigenvalues: max Re, min damping ratio

@@ -54,6 +54,25 @@ def test_eigen_screen_at_window_edges(n_gen, prec):
             assert abs(got["min_zeta"][q] - ref["min_zeta"]) <= 1e-6, q
 
 
+# state orders 59, 64, 84, 109 (and 5 less with a unit out) around the blocks of 60 from which the FP32 QR
+# runs two sweeps at a time, 48 steps apart
+@pytest.mark.parametrize("n_gen", [12, 13, 17, 22])
+@pytest.mark.parametrize("prec", [cs.PREC_FP64, cs.PREC_MIXED], ids=["fp64", "mixed"])
+def test_two_sweeps_at_a_time(n_gen, prec):
+    net = synth.make_network(24, 36, n_gen, 20, 1, seed=5, levels=(0.3,))
+    ei, ej = [-1, 0, 4, net.n_branch + n_gen - 1, 9], [-1, -1, -1, -1, 13]
+    ctx = cs.Context(precision=prec)
+    got = _run(ctx, ctx.load_network(net), ei, ej)
+    reruns = ctx.eigen_reruns()
+    ctx.close()
+    for q in range(len(ei)):
+        ref = pipeline.evaluate(net, 0, ei[q], ej[q])
+        assert int(got["klass"][q]) == ref["klass"]
+        assert abs(got["max_re"][q] - ref["max_re"]) <= 1e-6, q
+        assert abs(got["min_zeta"][q] - ref["min_zeta"]) <= 1e-6, q
+    assert reruns == 0
+
+
 @pytest.mark.parametrize("mode", [cs.RISK_EQ3, cs.RISK_ORDERED])
 @pytest.mark.parametrize("n_samples", [1, 2, 31, 32, 33, 65])
 def test_batched_risk_index_at_tile_edges(n_samples, mode):
