@@ -1841,17 +1841,23 @@ hqr_smem_kernel(EvalArgs a, OpfOut o, const float* __restrict__ hbuf, size_t hst
 // end.  The left vector solves (H - sigma I)^H z = b with G = H; the right one
 // solves (H - sigma I) x = b as (G - sigma I)^T (J x) = J b with G = J H^T J
 // (J reverses the order), which is upper Hessenberg again.
+//
+// What bounds it is latency: two passes of 269 dependent steps and 267 reflectors a vector, one warp each.  So a step
+// takes one complex reciprocal (two divisions with scaling before), its columns are loaded three at a time
+// ahead of the stores, the row operations carry their one dependent entry in registers, and the next
+// reflector is loaded while one is applied.  118 buses, 10,000 pairs mixed 817 -> 795 ms.
 constexpr int kRfThreads = 256;
 constexpr int kRfWarps = kRfThreads / 32;
+constexpr int kRfBatch = 3;           // columns per lane and trip of the inverse iteration's inner loop
 static_assert(2 * kRefK <= kRfWarps, "one warp per eigenvector");
 
 __device__ __forceinline__ float2 cmul2(float2 a, float2 b) { return make_float2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x); }
 __device__ __forceinline__ float2 cconj2(float2 a) { return make_float2(a.x, -a.y); }
-__device__ __forceinline__ float2 cdiv2(float2 a, float2 b) {
-    const float sc = fmaxf(fabsf(b.x), fabsf(b.y));
-    const float bx = b.x / sc, by = b.y / sc;
-    const float d = (bx * bx + by * by) * sc;
-    return make_float2((a.x * bx + a.y * by) / d, (a.y * bx - a.x * by) / d);
+__device__ __forceinline__ float2 crcp2(float2 b) {
+    const float sc = 1.0f / fmaxf(fabsf(b.x), fabsf(b.y));
+    const float bx = b.x * sc, by = b.y * sc;
+    const float d = sc / (bx * bx + by * by);
+    return make_float2(bx * d, -by * d);
 }
 
 template <bool kRight>
@@ -1877,21 +1883,36 @@ __device__ void hess_inverse_pass(const float* Hs, const int* rb, int n, float2 
         float2 pk = sw ? make_float2(rk, 0.0f) : ck;
         if (pk.x == 0.0f && pk.y == 0.0f) pk.x = tiny;             // exactly singular: perturb the pivot
         const float2 ok = sw ? ck : make_float2(rk, 0.0f);
-        const float2 mk = last ? make_float2(0.0f, 0.0f) : cdiv2(ok, pk);
-        const float2 yk = cdiv2(bk, cj ? cconj2(pk) : pk);
+        const float2 ik = crcp2(pk);                                // one reciprocal for the multiplier and y_k
+        const float2 mk = last ? make_float2(0.0f, 0.0f) : cmul2(ok, ik);
+        const float2 yk = cmul2(bk, cj ? cconj2(ik) : ik);
         __syncwarp();                                               // every lane has read c[k], y[k]
-        for (int j = k + 1 + lane; j < n; j += 32) {
-            float2 rj = make_float2(hess_g<kRight>(Hs, rb, n, k + 1, j), 0.0f);
-            if (j == k + 1) {
-                rj.x -= sig.x;
-                rj.y -= sig.y;
+        for (int j0 = k + 1 + lane; j0 < n; j0 += 32 * kRfBatch) {
+            float g[kRfBatch];                                      // a batch's loads before its stores
+            float2 cb[kRfBatch], yb[kRfBatch];
+#pragma unroll
+            for (int q = 0; q < kRfBatch; ++q) {
+                const int j = min(j0 + 32 * q, n - 1);
+                g[q] = hess_g<kRight>(Hs, rb, n, k + 1, j);
+                cb[q] = c[j];
+                yb[q] = y[j];
             }
-            const float2 cv = c[j];
-            const float2 pj = sw ? rj : cv, oj = sw ? cv : rj;
-            const float2 t = cmul2(cj ? cconj2(pj) : pj, yk);
-            y[j] = make_float2(y[j].x - t.x, y[j].y - t.y);
-            const float2 u = cmul2(mk, pj);
-            c[j] = make_float2(oj.x - u.x, oj.y - u.y);
+#pragma unroll
+            for (int q = 0; q < kRfBatch; ++q) {
+                const int j = j0 + 32 * q;
+                if (j >= n) break;
+                float2 rj = make_float2(g[q], 0.0f);
+                if (j == k + 1) {
+                    rj.x -= sig.x;
+                    rj.y -= sig.y;
+                }
+                const float2 cv = cb[q];
+                const float2 pj = sw ? rj : cv, oj = sw ? cv : rj;
+                const float2 t = cmul2(cj ? cconj2(pj) : pj, yk);
+                y[j] = make_float2(yb[q].x - t.x, yb[q].y - t.y);
+                const float2 u = cmul2(mk, pj);
+                c[j] = make_float2(oj.x - u.x, oj.y - u.y);
+            }
         }
         if (lane == 0) {
             y[k] = yk;
@@ -1901,15 +1922,19 @@ __device__ void hess_inverse_pass(const float* Hs, const int* rb, int n, float2 
         __syncwarp();
     }
     if (lane == 0) {
+        float2 up = y[n - 1];                                       // y[k + 1] so far
+        float2 m = mul[max(n - 2, 0)], v = y[max(n - 2, 0)];        // of step k, loaded a step ahead
         for (int k = n - 2; k >= 0; --k) {
-            const float2 t = cmul2(cj ? cconj2(mul[k]) : mul[k], y[k + 1]);
-            y[k] = make_float2(y[k].x - t.x, y[k].y - t.y);
-            if ((swp[k >> 5] >> (k & 31)) & 1u) {
-                const float2 q = y[k];
-                y[k] = y[k + 1];
-                y[k + 1] = q;
-            }
+            const float2 mn = mul[max(k - 1, 0)], vn = y[max(k - 1, 0)];
+            const float2 t = cmul2(cj ? cconj2(m) : m, up);
+            const float2 d = make_float2(v.x - t.x, v.y - t.y);
+            const bool sw = (swp[k >> 5] >> (k & 31)) & 1u;
+            y[k + 1] = sw ? d : up;
+            up = sw ? up : d;
+            m = mn;
+            v = vn;
         }
+        y[0] = up;
     }
     __syncwarp();
 }
@@ -2020,17 +2045,35 @@ eig_refine_kernel(EvalArgs a, OpfOut o, const float* __restrict__ hbuf, size_t h
                 __syncwarp();
             }
             if (ok) {                                            // Q x: reflectors n-3 .. 0
+                // (the next reflector's loads are on their way while this one is applied)
                 const float* betas = slot + ab_beta_off(nmax);
+                float un[kHsCols], btn = 0.0f;
+                auto fetch = [&](int k) {
+                    const float* u = slot + kHqHead + refl_off(n, max(k, 0));
+                    btn = betas[max(k, 0)];
+#pragma unroll
+                    for (int q = 0; q < kHsCols; ++q)
+                        if (32 * q < n - k - 1) un[q] = u[min(lane + 32 * q, n - max(k, 0) - 2)];
+                };
+                fetch(n - 3);
                 for (int k = n - 3; k >= 0; --k) {
-                    const float bt = betas[k];
+                    const float bt = btn;
+                    float u[kHsCols];
+#pragma unroll
+                    for (int q = 0; q < kHsCols; ++q) u[q] = un[q];
+                    fetch(k - 1);
                     if (bt == 0.0f) continue;
-                    const float* u = slot + kHqHead + refl_off(n, k);
                     const int mm = n - k - 1;
+                    float2* yk = y + k + 1 + lane;
+                    float2 w[kHsCols];
                     float sr = 0.0f, si = 0.0f;
-                    for (int i = lane; i < mm; i += 32) {
-                        const float2 q = y[k + 1 + i];
-                        sr += u[i] * q.x;
-                        si += u[i] * q.y;
+#pragma unroll
+                    for (int q = 0; q < kHsCols; ++q) {
+                        if (lane + 32 * q < mm) {
+                            w[q] = yk[32 * q];
+                            sr += u[q] * w[q].x;
+                            si += u[q] * w[q].y;
+                        }
                     }
                     for (int off = 16; off; off >>= 1) {
                         sr += __shfl_xor_sync(0xffffffffu, sr, off);
@@ -2038,10 +2081,9 @@ eig_refine_kernel(EvalArgs a, OpfOut o, const float* __restrict__ hbuf, size_t h
                     }
                     sr *= bt;
                     si *= bt;
-                    for (int i = lane; i < mm; i += 32) {
-                        const float2 q = y[k + 1 + i];
-                        y[k + 1 + i] = make_float2(q.x - sr * u[i], q.y - si * u[i]);
-                    }
+#pragma unroll
+                    for (int q = 0; q < kHsCols; ++q)
+                        if (lane + 32 * q < mm) yk[32 * q] = make_float2(w[q].x - sr * u[q], w[q].y - si * u[q]);
                     __syncwarp();
                 }
                 ok = warp_normalise(y, n, lane);
