@@ -26,6 +26,20 @@ CS_HD cplx cdiv(cplx a, cplx b) {
     return cplx{(a.re * b.re + a.im * b.im) / d, (a.im * b.re - a.re * b.im) / d};
 }
 
+// Opens a kernel's dynamic shared memory to all that a block may have beside its static memory.  The attribute
+// belongs to the function on the device, not to a context: a call that set it to its own size could lower it
+// between another context's setting and launch, and that launch would fail.
+inline cudaError_t open_shared(const void* kernel) {
+    int dev = 0, optin = 0;
+    cudaFuncAttributes fa{};
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, kernel);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, optin - (int)fa.sharedSizeBytes);
+    return e;
+}
+
 // ----------------------------------------------------- device network data ----
 // All arrays are device pointers owned by the library (one allocation per net).
 struct DevNet {

@@ -2242,7 +2242,7 @@ static cudaError_t launch_mode(const DevNet& net, const EvalArgs& a, OpfOut o, d
                                int sms, int* counter, cudaStream_t s) {
     const size_t smem = sizeof(double) * ((size_t)((net.ng + 1) >> 1) + 15 * (size_t)net.ng);
     if (smem > 48 * 1024) {
-        cudaError_t e = cudaFuncSetAttribute(dyn_kernel<kMode>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        cudaError_t e = open_shared((const void*)dyn_kernel<kMode>);
         if (e != cudaSuccess) return e;
     }
     // One block has a chain of dependent FP64 steps (the QR bulge, one warp) between wide phases: with
@@ -2277,21 +2277,21 @@ cudaError_t launch_dyn(const DevNet& net, const EvalArgs& a, OpfOut o, double da
         if (e != cudaSuccess) return e;
         const int nmax = 5 * net.ng - 1;
         const size_t hsm = hess_smem_bytes(nmax);
-        e = cudaFuncSetAttribute(hess_cluster_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)hsm);
+        e = open_shared((const void*)hess_cluster_kernel);
         if (e != cudaSuccess) return e;
         const int gh = 2 * (int)std::min<int64_t>((int64_t)std::max(1, sms / 2), a.n);
         hess_cluster_kernel<<<gh, kHsThreads, hsm, s>>>(a, o, abuf, astride, hbuf, hstride, nmax, counters + 3);
         e = cudaGetLastError();
         if (e != cudaSuccess) return e;
         const size_t qsm = qr_smem_bytes(nmax);
-        e = cudaFuncSetAttribute(hqr_smem_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)qsm);
+        e = open_shared((const void*)hqr_smem_kernel);
         if (e != cudaSuccess) return e;
         const int gq = (int)std::min<int64_t>((int64_t)sms, a.n);
         hqr_smem_kernel<<<gq, kQrThreads, qsm, s>>>(a, o, hbuf, hstride, nmax, damping_min, cand, counters + 1);
         e = cudaGetLastError();
         if (e != cudaSuccess) return e;
         const size_t rsm = refine_smem_bytes(nmax);
-        e = cudaFuncSetAttribute(eig_refine_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)rsm);
+        e = open_shared((const void*)eig_refine_kernel);
         if (e != cudaSuccess) return e;
         eig_refine_kernel<<<gq, kRfThreads, rsm, s>>>(a, o, hbuf, hstride, abuf, astride, a64, dyn_a64_stride(net),
                                                        cand, nmax, damping_min, counters + 4);

@@ -122,7 +122,7 @@ cudaError_t launch_islands(const DevNet& net, const EvalArgs& a, int* islanded, 
     const size_t smem = per_warp * wpb;
     if (smem > (size_t)optin) return cudaErrorInvalidValue;     // one bus array alone does not fit
     if (smem > 48 * 1024) {
-        e = cudaFuncSetAttribute(islands_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        e = open_shared((const void*)islands_kernel);
         if (e != cudaSuccess) return e;
     }
     int blocks = (a.n + wpb - 1) / wpb;

@@ -297,7 +297,7 @@ cudaError_t launch_risk_batch(int nE, const uint8_t* S1, const uint8_t* S2, cons
     const int rows = (nE + parts - 1) / parts;
     const size_t smem = sizeof(double) * kTile * (size_t)(nE | 1) + sizeof(unsigned) * (size_t)rows * ((nE + 31) / 32);
     if (ns >= kRiskTileMin && tiles <= 0x7fffffffll && smem + 1024 <= (size_t)optin) {
-        e = cudaFuncSetAttribute(risk_tile_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        e = open_shared((const void*)risk_tile_kernel);
         if (e != cudaSuccess) return e;
         risk_tile_kernel<<<dim3((unsigned)tiles, (unsigned)((nE + rows - 1) / rows)), 256, smem, s>>>(
             nE, rows, S1, S2, lam, ns, mode, R, err, bad_bit);

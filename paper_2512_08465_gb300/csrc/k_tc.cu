@@ -422,7 +422,7 @@ cudaError_t launch_hess_tc(int batch, int n, float* A, long long sA, float* ws, 
     if (batch <= 0 || n < 3) return cudaSuccess;
     const size_t wss = hess_ws_floats(n);
     const size_t csm = sizeof(float) * (size_t)n;
-    cudaError_t e = cudaFuncSetAttribute(hess_col_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)csm);
+    cudaError_t e = open_shared((const void*)hess_col_kernel);
     if (e != cudaSuccess) return e;
     // workspace views of the first matrix for the tensor-core products (layout of hess_ws)
     const long long sW = (long long)wss;
