@@ -478,15 +478,22 @@ __device__ __forceinline__ bool qr_safe(double x) {
     return (unsigned)((__double2hiint(x) >> 20) - (1023 - 99)) <= 2u * 99u;
 }
 
-// matrices: row-major in global memory, packed Hessenberg rows in shared memory
+// matrices: row-major in global memory, packed Hessenberg rows in shared memory.  Wide: the type in which
+// a sweep's shifts, its first column and its reflectors are formed before they are rounded to T.  FP64 for
+// a matrix in global memory in both forms: the FP32 eigenvalues of a large network are its record (there is no
+// refinement behind them).  600 pairs of 300 buses against their FP64 form: 3.0e-6 at most and 6.5e-7 on
+// average, with all of it in FP32 3.3e-6 and 7.1e-7; one scenario takes 123 ms instead of 83, 600 pairs 264
+// instead of 255.
 template <typename T>
 struct DenseMat {
+    using Wide = double;
     T* a;
     int n;
     __device__ T* at(int i, int j) const { return a + (size_t)i * n + j; }
 };
 template <typename T>
 struct PackedMat {
+    using Wide = T;
     T* a;
     const int* rb;
     __device__ T* at(int i, int j) const { return a + rb[i] + j; }
@@ -531,9 +538,10 @@ __device__ __forceinline__ QrRefl<T> qr_reflector(T x0, T x1, T x2) {
 
 // The bulge between two steps: the entries of its column k - 1 (x, rows k .. k + 2) and the one it
 // fills in column k (b, row k + 2).  They live in registers, never in the matrix.
-template <typename T>
+template <typename T, typename R>
 struct QrBulge {
-    T x0, x1, x2, b;
+    R x0, x1, x2;
+    T b;
 };
 
 // Reflectors first .. cnt - 1 on the entries y of one row or column.
@@ -561,7 +569,9 @@ __device__ __forceinline__ void qr_apply(T (&y)[kQrNB<T> + 2], const QrSpace<T>&
 // lane keeps: rows k .. k + 2 of columns k and k + 1, and column k + 2, fetched before the reflector
 // is known.  An FP64 instruction takes longer than a shuffle, so there the entries are fetched.
 template <typename T, typename M>
-__device__ __forceinline__ void qr_chase_full(const M& A, int lo, int hi, int kw, QrBulge<T>& bu, QrSpace<T>& sp) {
+__device__ __forceinline__ void qr_chase_full(const M& A, int lo, int hi, int kw, QrBulge<T, typename M::Wide>& bu,
+                                              QrSpace<T>& sp) {
+    using R = typename M::Wide;
     constexpr int NB = kQrNB<T>;
     constexpr bool kCopies = sizeof(T) == 4;
     const unsigned all = 0xffffffffu;
@@ -571,7 +581,8 @@ __device__ __forceinline__ void qr_chase_full(const M& A, int lo, int hi, int kw
     for (int r = 0; r < NB + 3; ++r)
         w[r] = (col <= hi && lane + 1 >= r) ? *A.at(kw + r, col) : (T)0;
     if (lane == 0) w[2] = bu.b;
-    T x0 = bu.x0, x1 = bu.x1, x2 = bu.x2, sub = 0;        // sub: subdiagonal entry (kw + lane, kw + lane - 1)
+    R x0 = bu.x0, x1 = bu.x1, x2 = bu.x2;
+    T sub = 0;                                            // subdiagonal entry (kw + lane, kw + lane - 1)
     T m00 = 0, m01 = 0, m10 = 0, m11 = 0, m20 = 0, m21 = 0;
     if (kCopies) {
         m00 = __shfl_sync(all, w[0], 0); m01 = __shfl_sync(all, w[0], 1);
@@ -587,10 +598,10 @@ __device__ __forceinline__ void qr_chase_full(const M& A, int lo, int hi, int kw
             c2 = __shfl_sync(all, w[t + 2], t + 2);
             s3 = __shfl_sync(all, w[t + 3], t + 2);
         }
-        const QrRefl<T> h = qr_reflector(x0, x1, x2);
-        const T v1 = h.v1, v2 = h.v2, tau = h.tau, t1 = tau * v1, t2 = tau * v2;
+        const QrRefl<R> h = qr_reflector(x0, x1, x2);
+        const T v1 = (T)h.v1, v2 = (T)h.v2, tau = (T)h.tau, t1 = (T)(h.tau * h.v1), t2 = (T)(h.tau * h.v2);
         sp.st[t] = {v1, v2, tau, t1, t2};                         // the same from every lane
-        if (lane == t) sub = h.alpha;
+        if (lane == t) sub = (T)h.alpha;
         T da, db, dc;
         if (kCopies) {
             const T d0 = m00 + v1 * m10 + v2 * m20, d1 = m01 + v1 * m11 + v2 * m21, d2 = c0 + v1 * c1 + v2 * c2;
@@ -630,7 +641,7 @@ __device__ __forceinline__ void qr_chase_full(const M& A, int lo, int hi, int kw
             x2 = __shfl_sync(all, w[t + 3], t);
         }
     }
-    bu = QrBulge<T>{x0, x1, x2, kCopies ? m20 : __shfl_sync(all, w[NB + 2], NB)};
+    bu = QrBulge<T, R>{x0, x1, x2, kCopies ? m20 : __shfl_sync(all, w[NB + 2], NB)};
     // a column of the window is final on and above its diagonal; its subdiagonal entry is the next
     // step's alpha (the last one's, the next window's, or x0 at the end of the sweep)
 #pragma unroll
@@ -648,7 +659,9 @@ __device__ __forceinline__ void qr_chase_full(const M& A, int lo, int hi, int kw
 // 4.4 ms.  Everything rolled: 15.0 and 4.9).
 constexpr int kQrUnroll = 4;
 template <typename T, typename M>
-__device__ __forceinline__ void qr_chase(const M& A, int lo, int hi, int kw, int cnt, QrBulge<T>& bu, QrSpace<T>& sp) {
+__device__ __forceinline__ void qr_chase(const M& A, int lo, int hi, int kw, int cnt, QrBulge<T, typename M::Wide>& bu,
+                                         QrSpace<T>& sp) {
+    using R = typename M::Wide;
     constexpr int NB = kQrNB<T>, U = kQrUnroll;
     static_assert(NB % U == 0 && U >= 3, "");
     constexpr bool kCopies = sizeof(T) == 4;
@@ -666,7 +679,8 @@ __device__ __forceinline__ void qr_chase(const M& A, int lo, int hi, int kw, int
 #pragma unroll
     for (int r = 0; r < U + 3; ++r) w[r] = load(r);
     if (lane == 0) w[2] = bu.b;
-    T x0 = bu.x0, x1 = bu.x1, x2 = bu.x2, sub = 0;        // sub: subdiagonal entry (kw + lane, kw + lane - 1)
+    R x0 = bu.x0, x1 = bu.x1, x2 = bu.x2;
+    T sub = 0;                                            // subdiagonal entry (kw + lane, kw + lane - 1)
     T m00 = 0, m01 = 0, m10 = 0, m11 = 0, m20 = 0, m21 = 0;
     if (kCopies) {
         m00 = __shfl_sync(all, w[0], 0); m01 = __shfl_sync(all, w[0], 1);
@@ -689,10 +703,10 @@ __device__ __forceinline__ void qr_chase(const M& A, int lo, int hi, int kw, int
                 c2 = __shfl_sync(all, w[u + 2], t + 2);
                 s3 = __shfl_sync(all, w[u + 3], t + 2);
             }
-            const QrRefl<T> h = qr_reflector(x0, x1, x2);
-            const T v1 = h.v1, v2 = h.v2, tau = h.tau, t1 = tau * v1, t2 = tau * v2;
+            const QrRefl<R> h = qr_reflector(x0, x1, x2);
+            const T v1 = (T)h.v1, v2 = (T)h.v2, tau = (T)h.tau, t1 = (T)(h.tau * h.v1), t2 = (T)(h.tau * h.v2);
             sp.st[t] = {v1, v2, tau, t1, t2};             // the same from every lane
-            if (lane == t) sub = h.alpha;
+            if (lane == t) sub = (T)h.alpha;
             T da, db, dc;
             if (kCopies) {
                 const T d0 = m00 + v1 * m10 + v2 * m20, d1 = m01 + v1 * m11 + v2 * m21, d2 = c0 + v1 * c1 + v2 * c2;
@@ -740,11 +754,11 @@ __device__ __forceinline__ void qr_chase(const M& A, int lo, int hi, int kw, int
         for (int u = 0; u < U; ++u) w[u + 3] = next[u];
     }
     const int end = (cnt + U - 1) / U * U;
-    bu = QrBulge<T>{x0, x1, x2, kCopies ? m20 : __shfl_sync(all, w[2], NB)};   // (the last window's is not used)
+    bu = QrBulge<T, R>{x0, x1, x2, kCopies ? m20 : __shfl_sync(all, w[2], NB)};   // (the last window's is not used)
 #pragma unroll
     for (int r = 0; r < 3; ++r) store(end + r, w[r]);
     if (lane < cnt && col > lo) *A.at(col, col - 1) = sub;
-    if (kw + cnt == hi && lane == 0) *A.at(hi, hi - 1) = x0;
+    if (kw + cnt == hi && lane == 0) *A.at(hi, hi - 1) = (T)x0;
 }
 
 // One window's strips: its reflectors on 32 of the rows above it and its own (each from its own step
@@ -800,24 +814,24 @@ struct QrStrips {
 // and product, a block whose eigenvalues differ by little (the exciters' cluster near -1/T_A) loses
 // the differences to cancellation in FP32 and its sweeps go nowhere (118 buses: 331 -> 276 sweeps a
 // scenario, and the scenario in 20,000 that ran to the sweep limit converges).
-template <typename T>
+template <typename R>
 struct QrShift {
-    T a11, a22, w;                               // trailing 2x2 block: diagonal, product of the off-diagonal
+    R a11, a22, w;                               // trailing 2x2 block: diagonal, product of the off-diagonal
 };
-template <typename T, typename M>
-__device__ __forceinline__ QrShift<T> qr_shift(const M& A, int hi, bool exceptional) {
-    QrShift<T> q{*A.at(hi - 1, hi - 1), *A.at(hi, hi), *A.at(hi - 1, hi) * *A.at(hi, hi - 1)};
+template <typename R, typename M>
+__device__ __forceinline__ QrShift<R> qr_shift(const M& A, int hi, bool exceptional) {
+    QrShift<R> q{(R)*A.at(hi - 1, hi - 1), (R)*A.at(hi, hi), (R)*A.at(hi - 1, hi) * (R)*A.at(hi, hi - 1)};
     if (exceptional) {
-        const T ww = fabs(*A.at(hi, hi - 1)) + fabs(*A.at(hi - 1, hi - 2));
-        q.a11 = q.a22 = q.a22 + (T)0.75 * ww;
-        q.w = (T)-0.4375 * ww * ww;
+        const R ww = fabs((R)*A.at(hi, hi - 1)) + fabs((R)*A.at(hi - 1, hi - 2));
+        q.a11 = q.a22 = q.a22 + (R)0.75 * ww;
+        q.w = (R)-0.4375 * ww * ww;
     }
     return q;
 }
-template <typename T, typename M>
-__device__ __forceinline__ void qr_start(const M& A, int lo, const QrShift<T>& q, QrBulge<T>& bu) {
-    const T h00 = *A.at(lo, lo), h01 = *A.at(lo, lo + 1), h10 = *A.at(lo + 1, lo), h11 = *A.at(lo + 1, lo + 1);
-    const T r = q.a22 - h00, s = q.a11 - h00;
+template <typename T, typename R, typename M>
+__device__ __forceinline__ void qr_start(const M& A, int lo, const QrShift<R>& q, QrBulge<T, R>& bu) {
+    const R h00 = *A.at(lo, lo), h01 = *A.at(lo, lo + 1), h10 = *A.at(lo + 1, lo), h11 = *A.at(lo + 1, lo + 1);
+    const R r = q.a22 - h00, s = q.a11 - h00;
     bu.x0 = (r * s - q.w) / h10 + h01;
     bu.x1 = h11 - h00 - r - s;
     bu.x2 = *A.at(lo + 2, lo + 1);
@@ -849,13 +863,14 @@ constexpr int kQrPair = 60;
 template <bool kTwo, typename T, typename M>
 __device__ __forceinline__ void qr_sweep(const M& A, int lo, int hi, bool exceptional, bool two,
                                          QrSpace<T> (&sp)[2][2], int nthreads) {
+    using R = typename M::Wide;
     constexpr int NB = kQrNB<T>;
     const int sweeps = kTwo && two ? 2 : 1;
     const int warp = threadIdx.x >> 5, nworkers = (nthreads >> 5) - sweeps;
     const int last = hi + (sweeps - 1) * kQrLag<T>;
-    QrBulge<T> bu{};
-    QrShift<T> q{};
-    if (warp < sweeps) q = qr_shift<T>(A, hi, exceptional);
+    QrBulge<T, R> bu{};
+    QrShift<R> q{};
+    if (warp < sweeps) q = qr_shift<R>(A, hi, exceptional);
     int par = 0;
     for (int ka = lo;; ka += NB, par ^= 1) {                      // (the last round: strips only)
         const int kw = ka - warp * kQrLag<T>;                     // of a chasing warp
@@ -894,10 +909,11 @@ __device__ __forceinline__ void qr_sweep(const M& A, int lo, int hi, bool except
 // sh.fail = 2 if it does not converge in 30 n sweeps.
 template <typename T>
 __device__ __noinline__ void hqr_global(T* Ag, const int n, double* wr, double* wi, DShared& sh) {
+    static_assert(sizeof(typename DenseMat<T>::Wide) == 8, "no refinement follows: shifts and reflectors in FP64");
     __shared__ QrSpace<T> sp[2][2];
     const int tid = threadIdx.x, nthr = blockDim.x;
     const DenseMat<T> A{Ag, n};
-    const T eps = (sizeof(T) == 8) ? (T)kEps : (T)kDeflTol;              // deflation tolerance
+    const double eps = (sizeof(T) == 8) ? kEps : (double)kDeflTol;       // deflation tolerance
     double hmax;
     {
         double hm = 0.0;
@@ -910,9 +926,9 @@ __device__ __noinline__ void hqr_global(T* Ag, const int n, double* wr, double* 
         // top of the unreduced block ending at hi: largest l <= hi with a negligible A[l][l-1]
         int cand = 0;
         for (int l = 1 + tid; l <= hi; l += nthr) {
-            T sd = fabs(*A.at(l - 1, l - 1)) + fabs(*A.at(l, l));
-            if (sd == (T)0) sd = (T)hmax;
-            if (fabs(*A.at(l, l - 1)) <= eps * sd) cand = max(cand, l);
+            double sd = fabs((double)*A.at(l - 1, l - 1)) + fabs((double)*A.at(l, l));
+            if (sd == 0.0) sd = hmax;
+            if (fabs((double)*A.at(l, l - 1)) <= eps * sd) cand = max(cand, l);
         }
         const int lo = bmax_int(sh, cand);
         if (lo == hi) {
