@@ -87,7 +87,8 @@ typedef struct {
                                   network's workspaces would pass ~6 GB) */
     int32_t precision;         /* CS_PREC_FP64 (default) or CS_PREC_MIXED */
     int64_t hbm_budget;        /* device bytes the context may hold (networks, workspaces,
-                                  request buffers); 0 = no limit */
+                                  request buffers); 0 = no limit (a workspace of a network from about
+                                  240 buses on then takes up to 2 GB of scratch where that is faster) */
     int32_t serve_slots;       /* batches in flight on the serving path (1..8, default 3) */
     int32_t batch_cap;         /* scenarios per serving batch (default 4096; larger requests are
                                   split over batches) */

@@ -54,7 +54,7 @@ int cap_dyn_of(const cs_ctx* ctx, const Network& net) {
     if (ctx->opt.ctas_per_sm > 0) return ctx->opt.ctas_per_sm;
     return net.dyn_cap > 0 ? net.dyn_cap : dyn_ctas_per_sm();
 }
-Grids grids(const cs_ctx* ctx, const Network& net, int64_t cn) {
+Grids grids(const cs_ctx* ctx, const Network& net, int64_t cn, bool tight = false) {
     // persistent kernels sized from occupancy, capped per SM (the network's tuned shape, if any)
     const DevNet& dn = net.dev;
     const int cap_opf = cap_opf_of(ctx, net);
@@ -65,13 +65,14 @@ Grids grids(const cs_ctx* ctx, const Network& net, int64_t cn) {
     g.per_opf = opf_scratch_doubles(dn);
     g.per_dyn = dyn_scratch_doubles(dn);
     if (ctx->opt.ctas_per_sm <= 0 && net.dyn_cap <= 0) {
-        // The OPF scratch (or two small-signal CTAs per SM) sets the workspace.  The default of four
-        // may exceed it up to kDynScratch, unless the device memory is budgeted: on 300 buses the four
-        // need 1.35 GB for the two's 0.74 GB, on 1,000 buses 14.7 GB for 7.4 GB (two there).
-        const size_t two = g.per_dyn * (size_t)std::min<int64_t>((int64_t)ctx->sms * 2, cn);
-        size_t lim = std::max(g.per_opf * g.g_opf, two);
-        if (ctx->opt.hbm_budget <= 0) lim = std::max(lim, kDynScratch / sizeof(double));
-        g.g_dyn = (int)std::min<size_t>(g.g_dyn, std::max<size_t>(1, lim / std::max<size_t>(1, g.per_dyn)));
+        // Four small-signal blocks per SM where their scratch is within the OPF's or two blocks', or within
+        // kDynScratch (not with a budget, nor after that much could not be allocated); else two, never between
+        // (launch_mode gives two blocks per SM twice the threads).  300 buses, 600 pairs: 1.35 GB and 472 ms
+        // with four, 0.74 GB and 554 ms with two (FP64 form; mixed 264 and 311 ms).
+        const int two = (int)std::max<int64_t>(1, std::min<int64_t>((int64_t)ctx->sms * 2, cn));
+        size_t lim = std::max(g.per_opf * g.g_opf, g.per_dyn * two);
+        if (ctx->opt.hbm_budget <= 0 && !tight) lim = std::max(lim, kDynScratch / sizeof(double));
+        if (g.per_dyn * g.g_dyn > lim) g.g_dyn = two;
     }
     return g;
 }
@@ -167,28 +168,43 @@ cs_status csi::evaluate_impl(cs_ctx* ctx, Workspace& ws, Network* net, int level
     const int nx = 2 * dn.nb + 2 * dn.ng;
     chunk = std::max<int64_t>(1, chunk);
     const int64_t cn = std::min<int64_t>(n, chunk);
-    const Grids gr = grids(ctx, *net, cn);
-    const int g_opf = gr.g_opf, g_dyn = gr.g_dyn;
-    const size_t per_opf = gr.per_opf, per_dyn = gr.per_dyn;
-    const size_t need = std::max(per_opf * g_opf, per_dyn * g_dyn) * sizeof(double);
-    CS_CUDA(ws.scratch.ensure(need));
-    CS_CUDA(ws.isl.ensure(sizeof(int) * cn));
-    CS_CUDA(ws.opfx.ensure(sizeof(double) * nx * cn));
-    CS_CUDA(ws.opfst.ensure(sizeof(int) * cn));
-    CS_CUDA(ws.counters.ensure(sizeof(int) * kCounters));
     // balanced and packed Hessenberg matrices between the kernels of the FP32 screen
     const bool split = split_path(ctx, dn);
-    if (split) {
-        CS_CUDA(ws.hbuf.ensure(sizeof(float) * dyn_hbuf_stride(dn) * cn));
-        CS_CUDA(ws.abuf.ensure(sizeof(float) * dyn_abuf_stride(dn) * cn));
-        CS_CUDA(ws.a64.ensure(sizeof(double) * dyn_a64_stride(dn) * cn));
-        CS_CUDA(ws.cand.ensure(sizeof(float) * dyn_cand_stride() * cn));
-    }
     const bool large = large_path(ctx, dn);
-    if (large) {
-        CS_CUDA(ws.abuf.ensure(sizeof(float) * dyn_abuf_stride(dn) * cn));
-        CS_CUDA(ws.hws.ensure(sizeof(float) * hess_tc_workspace_floats(5 * dn.ng - 1) * cn));
+    auto allocate = [&](const Grids& g) -> cudaError_t {
+        cudaError_t e = ws.scratch.ensure(std::max(g.per_opf * g.g_opf, g.per_dyn * g.g_dyn) * sizeof(double));
+        auto also = [&](DevBuf& b, size_t bytes) { if (e == cudaSuccess) e = b.ensure(bytes); };
+        also(ws.isl, sizeof(int) * cn);
+        also(ws.opfx, sizeof(double) * nx * cn);
+        also(ws.opfst, sizeof(int) * cn);
+        also(ws.counters, sizeof(int) * kCounters);
+        if (split) {
+            also(ws.hbuf, sizeof(float) * dyn_hbuf_stride(dn) * cn);
+            also(ws.abuf, sizeof(float) * dyn_abuf_stride(dn) * cn);
+            also(ws.a64, sizeof(double) * dyn_a64_stride(dn) * cn);
+            also(ws.cand, sizeof(float) * dyn_cand_stride() * cn);
+        }
+        if (large) {
+            also(ws.abuf, sizeof(float) * dyn_abuf_stride(dn) * cn);
+            also(ws.hws, sizeof(float) * hess_tc_workspace_floats(5 * dn.ng - 1) * cn);
+        }
+        return e;
+    };
+    Grids gr = grids(ctx, *net, cn, ws.tight);
+    cudaError_t got = allocate(gr);
+    if (got == cudaErrorMemoryAllocation) {            // once more with two small-signal blocks per SM, if that is less
+        const Grids less = grids(ctx, *net, cn, true);
+        if (less.g_dyn < gr.g_dyn) {
+            cudaGetLastError();
+            ws.tight = true;
+            ws.scratch.release();
+            gr = less;
+            got = allocate(gr);
+        }
     }
+    CS_CUDA(got);
+    const int g_opf = gr.g_opf, g_dyn = gr.g_dyn;
+    const size_t per_opf = gr.per_opf, per_dyn = gr.per_dyn;
     if (!ctx->err_word.p) {
         CS_CUDA(ctx->err_word.ensure(sizeof(int) * 2));
         CS_CUDA(cudaMemset(ctx->err_word.p, 0, sizeof(int) * 2));

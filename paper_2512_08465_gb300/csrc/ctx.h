@@ -69,6 +69,7 @@ struct Workspace {
     DevBuf scratch, isl, opfx, opfst, counters, hbuf, abuf, a64, cand, hws;
     cudaEvent_t free = nullptr;
     bool used = false;
+    bool tight = false;               // the scratch of four small-signal blocks per SM could not be allocated
     size_t bytes() const {
         return scratch.bytes + isl.bytes + opfx.bytes + opfst.bytes + counters.bytes + hbuf.bytes + abuf.bytes +
                a64.bytes + cand.bytes + hws.bytes;
