@@ -706,8 +706,11 @@ cs_status cs_network_stats(cs_ctx* ctx, int32_t net_id, int64_t* stats, int32_t 
     if (!stats || n_stats < 0) return fail(ctx, CS_E_ARG, "NULL stats");
     const DevNet& d = it->second->dev;
     const Symbolic& S = it->second->sym;
+    // (of a batch that fills the device: the default may be held to two by its scratch)
+    const int64_t cap = cap_dyn_of(ctx, *it->second);
+    const int64_t dyn_per_sm = grids(ctx, *it->second, ctx->sms * std::max<int64_t>(cap, opf_ctas_per_sm())).g_dyn / ctx->sms;
     const int64_t v[12] = {d.nb, d.nbr, d.ng, d.nL, (int64_t)S.upd_a.size(), d.nlevels, 5LL * d.ng - 1,
-                           (int64_t)it->second->nlev, cap_opf_of(ctx, *it->second), cap_dyn_of(ctx, *it->second),
+                           (int64_t)it->second->nlev, cap_opf_of(ctx, *it->second), dyn_per_sm,
                            (ctx->opt.ctas_per_sm == 0 && it->second->opf_cap > 0) ? 1 : 0, it->second->max_it};
     for (int i = 0; i < n_stats && i < 12; ++i) stats[i] = v[i];
     return CS_OK;

@@ -21,6 +21,15 @@ def _net(n_bus):
     return synth.case118() if n_bus == 118 else synth.case_scaled(n_bus, seed=n_bus, levels=(0.6,), vband=(0.85, 1.15))
 
 
+# 118 buses: within the OPF's scratch; 300: 1.35 GB for four, 0.74 GB budgeted; 520: 3.9 GB for four
+@pytest.mark.parametrize("n_bus,budget,blocks", [(118, 0, 4), (118, 64 << 30, 4), (300, 0, 4), (300, 64 << 30, 2),
+                                                 (520, 0, 2)])
+def test_blocks_per_sm(n_bus, budget, blocks):
+    ctx = cs.Context(hbm_budget=budget)
+    assert ctx.network_stats(ctx.load_network(_net(n_bus)))["dyn_ctas_per_sm"] == blocks
+    ctx.close()
+
+
 def test_short_device_memory():
     """600 pairs of 300 buses need 1.35 GB of scratch with four blocks per SM and 0.74 GB with two; with 1 GB free
     every record is as with all the memory, bit for bit (they do not depend on the shape)."""
