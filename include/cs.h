@@ -87,8 +87,8 @@ typedef struct {
                                   network's workspaces would pass ~6 GB) */
     int32_t precision;         /* CS_PREC_FP64 (default) or CS_PREC_MIXED */
     int64_t hbm_budget;        /* device bytes the context may hold (networks, workspaces,
-                                  request buffers); 0 = no limit (a workspace of a network from about
-                                  240 buses on then takes up to 2 GB of scratch where that is faster) */
+                                  request buffers); 0 = no limit (a workspace of a network of more than
+                                  256 buses then takes up to 2 GB of scratch where that is faster) */
     int32_t serve_slots;       /* batches in flight on the serving path (1..8, default 3) */
     int32_t batch_cap;         /* scenarios per serving batch (default 4096; larger requests are
                                   split over batches) */
@@ -135,8 +135,12 @@ typedef struct {
     uint8_t* klass;            /* CS_SECURE .. CS_EIG_FAIL */
     uint8_t* severe;           /* S_c in {0, 1} */
     int16_t* n_islands;        /* number of islands of the post-contingency network */
-    int16_t* opf_iters;        /* interior-point iterations taken (0 if not run); the cap for a scenario
-                                  stopped because it can no longer converge within it */
+    int16_t* opf_iters;        /* interior-point iterations taken (0 if not run).  The cap, without having
+                                  taken them, for an infeasible scenario whose complementarity is
+                                  so far above the tolerance that the iterations left could not bring
+                                  it down (unless a bus angle passed 2^100 rad); a run to the end
+                                  would state the cap too, or fewer if its Newton system became
+                                  singular or non-finite on the way */
     double* cost;              /* OPF cost, $/h (NaN if not converged) */
     double* max_re;            /* largest real part, structural zero mode removed (NaN if not run) */
     double* min_zeta;          /* smallest damping ratio (NaN if not run) */
