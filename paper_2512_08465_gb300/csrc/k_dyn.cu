@@ -651,7 +651,6 @@ __device__ __forceinline__ void qr_chase_full(const M& A, int lo, int hi, int kw
     if (lane < NB && col > lo) *A.at(col, col - 1) = sub;
 }
 
-//
 // qr_chase_full takes a window that ends three rows above the block's end or higher, unrolled; qr_chase any, in a
 // loop of kQrUnroll steps with the rows in a rolling buffer.  The size of the code counts: with all SMs at
 // it a warp waits for its instructions (118 buses, three scenarios on each SM: 15.0 ms with both kinds
@@ -970,8 +969,8 @@ __device__ void eigen_screen(T* A, const int n, T* cs, T* rs, T* v, T* part, dou
 
 // ---------------------------------------------------------------------------
 // Packed Hessenberg storage for the shared-memory QR: row i keeps columns
-// max(i-3, 0)..n-1 (the Hessenberg part plus the two sub-diagonals the bulge
-// passes through).  hq_off(n, i) is the offset of row i; hq_off(n, n) the size.
+// max(i-3, 0)..n-1: the Hessenberg part, and two sub-diagonals more that stay zero (a
+// sweep's bulge is in registers; the rows' offsets are those of a bulge in the matrix).  hq_off(n, i) is the offset of row i; hq_off(n, n) the size.
 __host__ __device__ inline int hq_start(int i) { return i > 3 ? i - 3 : 0; }
 __host__ __device__ inline int hq_off(int n, int i) {
     if (i <= 3) return n * i;

@@ -61,10 +61,7 @@ constexpr int kThreads = CS_OPF_THREADS;   // threads per scenario CTA
 constexpr int kCtasPerSm = CS_OPF_CTAS;    // resident CTAs per SM the register budget is sized for
 constexpr int kWarps = kThreads / 32;
 constexpr int kGroups = kThreads / 16;     // groups of 16 threads, one thread per entry of a 4x4 block
-#ifndef CS_OPF_BATCH
-#define CS_OPF_BATCH 4
-#endif
-constexpr int kBatch = CS_OPF_BATCH;       // block updates whose loads are in flight together
+constexpr int kBatch = 4;                  // block updates whose loads are in flight together
 constexpr int kRec = 34;     // doubles per branch record
 constexpr double kXi = 0.99995;
 constexpr double kSigma = 0.1;

@@ -282,10 +282,11 @@ risk_tile_kernel(int E, int rows, const uint8_t* __restrict__ S1, const uint8_t*
 cudaError_t launch_risk_batch(int nE, const uint8_t* S1, const uint8_t* S2, const double* lam, long long ns,
                               int mode, double* R, int* err, int bad_bit, cudaStream_t s) {
     if (nE <= 0 || ns <= 0) return cudaSuccess;
-    // A thread per sample where a tile of rates and the bit rows fit a quarter of an SM's shared memory
-    // (up to ~200 elements) or at least one block of it (~800); above, and for few samples (a tile would
-    // leave lanes and SMs idle: 240 elements, 8 samples 23.7 us against 20.4, 16 samples 26.1 against
-    // 26.6, 64 samples 29.5 against 59.2), a warp per sample.
+    // A thread per sample where a tile of rates and the bit rows fit a block's shared memory (up to ~900
+    // elements; four blocks an SM up to ~200); above, and for few samples (a tile would leave lanes and SMs idle:
+    // 240 elements, 8 samples 23.7 us against 20.4), a warp per sample.  16 samples, tile against warp: 25 elements
+    // 6.2 / 6.3 us, 120 elements 10.5 / 10.3, 240 elements 18.5 / 18.5, 790 elements 45 / 114; 64 samples: 6.3 /
+    // 16.5, 12.5 / 28.8, 20.7 / 57.6, 109 / 447.
     int dev = 0, sms = 0, optin = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
